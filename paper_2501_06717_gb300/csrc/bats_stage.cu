@@ -212,7 +212,7 @@ __global__ void k_cfl(const double* __restrict__ U, const float* __restrict__ Wt
       float Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
       float sf = 0.f;
       for (int e = 0; e < 3; e++) {
-        float cf = fast_speed_n<float>(float(ph.gamma), W[0], W[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
+        float cf = fast_speed_n(float(ph.gamma), W[0], W[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
         sf = sf + (fabsf(W[1 + e]) + cf) * rcp_approx(float(dxd[e]));
       }
       s = sf;
@@ -221,11 +221,8 @@ __global__ void k_cfl(const double* __restrict__ U, const float* __restrict__ Wt
       for (int v = 0; v < NV; v++) u[v] = U[base + v * NCELL];
       prim64(u, ph.gm1, W);
       if (ph.b0 != B0_NONE) b0_at<double>(ph, xc, B0c);
-      double Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
-      for (int e = 0; e < 3; e++) {
-        double cf = fast_speed_exact(ph.gamma, W[0], W[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
-        s = s + (fabs(W[1 + e]) + cf) / dxd[e];
-      }
+      const double Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
+      s = cfl_sum64(ph.gamma, W, Bt, G.idx[B.level]);
     }
   }
   // local time stepping: the cell's own dt (0 in the body)
@@ -371,7 +368,7 @@ __global__ void __launch_bounds__(64) k_reflux(const StageArgs a, const RefluxTa
       float sacc = 0.f;
 #pragma unroll
       for (int e = 0; e < 3; e++) {
-        const float cf = fast_speed_n<float>(ph.gammaf, Wn[0], Wn[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
+        const float cf = fast_speed_n(ph.gammaf, Wn[0], Wn[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
         sacc = sacc + (fabsf(Wn[1 + e]) + cf) * G.idxf[lev][e];
       }
       md = f2d_int(sacc);
@@ -384,13 +381,7 @@ __global__ void __launch_bounds__(64) k_reflux(const StageArgs a, const RefluxTa
         b0_face<double>(ph, -1, ci, cj, ck, gb0, gb1, gb2, G.lo[0], G.lo[1], G.lo[2], G.dx[lev][0], G.dx[lev][1],
                         G.dx[lev][2], B0c);
       const double Bt[3] = {B0c[0] + Wn[4], B0c[1] + Wn[5], B0c[2] + Wn[6]};
-      double sacc = 0.0;
-#pragma unroll
-      for (int e = 0; e < 3; e++) {
-        const double cf = fast_speed_exact(ph.gamma, Wn[0], Wn[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
-        sacc = sacc + (fabs(Wn[1 + e]) + cf) / G.dx[lev][e];
-      }
-      md = sacc;
+      md = cfl_sum64(ph.gamma, Wn, Bt, G.idx[lev]);
     }
     if (md > 0.0) atomicMax(&a.smax_next[B.grid], static_cast<unsigned long long>(__double_as_longlong(md)));
     if (a.dtc) a.dtc[static_cast<int64_t>(T.blk) * NCELL + c] = a.cfl / md;

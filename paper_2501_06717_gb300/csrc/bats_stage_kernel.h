@@ -143,6 +143,53 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 reciprocal and square roots from the hardware's estimates (PTX
+// rcp/rsqrt.approx.ftz.f64, about 20 bits, issued off the FP64 pipe) refined by
+// one third-order Newton step (Householder's method, order 2: the error cubed):
+// with e = 1 - x y,      1/x       = y (1 + e + e^2) + O(e^3);
+// with r = 1 - x y^2,    1/sqrt(x) = y (1 + r/2 + 3 r^2 / 8) + O(r^3).
+// The last operation is an FMA onto the leading term, so the results are within
+// about one unit in the last place.  GB300 issues 2 FP64 operations per clock
+// and SM: these take 3 and 5 of them where the general division and square root
+// take several times as many, and a face has two speeds of two roots each.
+__device__ __forceinline__ double rcp64(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(fma(e, e, e), y, y);
+}
+// The estimate of 1/sqrt(x); 0 for x = 0 or denormal, so that the roots below
+// give sqrt(0) = 0 (NaN for x < 0 or NaN).
+__device__ __forceinline__ double rsqrt64_est(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return static_cast<uint32_t>(__double2hiint(x)) < 0x00100000u ? 0.0 : y;
+}
+__device__ __forceinline__ double sqrt64(double x) {
+  const double y = rsqrt64_est(x), t = x * y;
+  const double r = fma(-t, y, 1.0);
+  return fma(fma(0.375, r, 0.5), r * t, t);
+}
+// a / sqrt(x)
+__device__ __forceinline__ double div_sqrt64(double a, double x) {
+  const double y = rsqrt64_est(x), c = a * y;
+  const double r = fma(-(x * y), y, 1.0);
+  return fma(fma(0.375, r, 0.5), r * c, c);
+}
+// Fast magnetosonic speed from half the sound term (gamma/2) p, half of B^2,
+// the squared normal field and rho:
+//   c_f^2 = (G + sqrt(G^2 - gamma p B_n^2)) / rho,  G = (gamma p + B^2) / 2,
+// the usual form with 1/rho taken out of both roots, which leaves no division
+// (c_f = Q / sqrt(Q rho)).
+__device__ __forceinline__ double fast_speed64(double gph, double hbsq, double bn2, double rho) {
+  const double G = gph + hbsq;
+  double D = fma(-2.0, gph * bn2, G * G);
+  D = __double2hiint(D) < 0 ? 0.0 : D;
+  const double Q = G + sqrt64(D);
+  return div_sqrt64(Q, Q * rho);
+}
+
+// ---------------------------------------------------------------------------
 // Precision-generic scalar ops.
 
 template <class R> struct Ops;
@@ -157,49 +204,25 @@ template <> struct Ops<float> {
   static __device__ __forceinline__ float abs_(float x) { return fabsf(x); }
 };
 
-template <class R>
-__device__ __forceinline__ R minmod_(R a, R b) {
-  R r = R(0);
-  r = (a > R(0) && b > R(0)) ? (a < b ? a : b) : r;
-  r = (a < R(0) && b < R(0)) ? (a > b ? a : b) : r;
-  return r;
-}
-// FP32: the smaller magnitude with a's sign when the signs agree, else 0 (a
-// zero argument gives a signed zero, which adds like 0), in five operations.
-template <>
-__device__ __forceinline__ float minmod_<float>(float a, float b) {
+// FP32 minmod: the smaller magnitude with a's sign when the signs agree, else
+// 0 (a zero argument gives a signed zero, which adds like 0), in five operations.
+__device__ __forceinline__ float minmod_f(float a, float b) {
   const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
   const float m = fminf(fabsf(a), fabsf(b));
   const float r = __uint_as_float((__float_as_uint(m) & 0x7fffffffu) | (ua & 0x80000000u));
   return static_cast<int32_t>(ua ^ ub) < 0 ? 0.f : r;
 }
-// MC limiter (beta = 2): sign(a) min(2|a|, 2|b|, |a+b|/2), 0 when signs differ.
-template <class R>
-__device__ __forceinline__ R mc_(R a, R b) {
-  R c = R(0.5) * (a + b);
-  R r = R(0);
-  if (a > R(0) && b > R(0)) {
-    R m = R(2) * a < R(2) * b ? R(2) * a : R(2) * b;
-    r = m < c ? m : c;
-  } else if (a < R(0) && b < R(0)) {
-    R m = R(2) * a > R(2) * b ? R(2) * a : R(2) * b;
-    r = m > c ? m : c;
-  }
-  return r;
-}
-// kind 0 minmod, 1 MC, 2 none (first order: piecewise-constant faces)
-// FP32: the same selection by the sign bits (2|a|, 2|b| and |a+b|/2 when the
-// signs agree, else 0).
-template <>
-__device__ __forceinline__ float mc_<float>(float a, float b) {
+// FP32 MC limiter (beta = 2): sign(a) min(2|a|, 2|b|, |a+b|/2), 0 when signs
+// differ, by the same selection on the sign bits.
+__device__ __forceinline__ float mc_f(float a, float b) {
   const uint32_t ua = __float_as_uint(a), ub = __float_as_uint(b);
   const float m = fminf(fminf(2.f * fabsf(a), 2.f * fabsf(b)), fabsf(0.5f * (a + b)));
   const float r = __uint_as_float((__float_as_uint(m) & 0x7fffffffu) | (ua & 0x80000000u));
   return static_cast<int32_t>(ua ^ ub) < 0 ? 0.f : r;
 }
-template <class R>
-__device__ __forceinline__ R limit_(int kind, R a, R b) {
-  return kind == 2 ? R(0) : (kind == 1 ? mc_(a, b) : minmod_(a, b));
+// kind 0 minmod, 1 MC, 2 none (first order: piecewise-constant faces)
+__device__ __forceinline__ float limit_(int kind, float a, float b) {
+  return kind == 2 ? 0.f : (kind == 1 ? mc_f(a, b) : minmod_f(a, b));
 }
 
 // Background field B0 at point x (split field B = B0 + B1).
@@ -226,13 +249,13 @@ __device__ __forceinline__ void b0_at(const PhysDev& ph, const R x[3], R B0[3]) 
 
 // Primitive recovery in FP64 (Eq. 5): u = m/rho, p = (gamma-1)(e1 - m.u/2 - B1.B1/2).
 __device__ __forceinline__ void prim64(const double U[8], double gm1, double W[8]) {
-  double rho = U[0];
-  double ux = U[1] / rho, uy = U[2] / rho, uz = U[3] / rho;
-  double ke = 0.5 * (U[1] * ux + U[2] * uy + U[3] * uz);
-  double me = 0.5 * (U[4] * U[4] + U[5] * U[5] + U[6] * U[6]);
-  W[0] = rho; W[1] = ux; W[2] = uy; W[3] = uz;
+  const double rinv = rcp64(U[0]);
+  const double ux = U[1] * rinv, uy = U[2] * rinv, uz = U[3] * rinv;
+  const double ke2 = fma(U[3], uz, fma(U[2], uy, U[1] * ux));
+  const double me2 = fma(U[6], U[6], fma(U[5], U[5], U[4] * U[4]));
+  W[0] = U[0]; W[1] = ux; W[2] = uy; W[3] = uz;
   W[4] = U[4]; W[5] = U[5]; W[6] = U[6];
-  W[7] = gm1 * ((U[7] - ke) - me);
+  W[7] = gm1 * fma(-0.5, me2, fma(-0.5, ke2, U[7]));
 }
 
 // Mixed form: FP32 primitives of an FP64 state.  The pressure comes from the
@@ -292,52 +315,48 @@ __device__ __forceinline__ void cons_from_prim(const R W[8], R inv_gm1, R U[8]) 
 }
 
 // Fast magnetosonic speed along the frame's normal (component 0) with total B.
-template <class R>
-__device__ __forceinline__ R fast_speed_n(R gamma, R rho, R p, R bx, R by, R bz) {
-  R rinv = Ops<R>::div_(R(1), rho);
-  R a2 = Ops<R>::div_(gamma * p, rho);
-  R b2 = (bx * bx + by * by + bz * bz) * rinv;
-  R bn2 = bx * bx * rinv;
-  R s = a2 + b2;
-  R disc = s * s - R(4) * a2 * bn2;
-  disc = disc < R(0) ? R(0) : disc;
-  return Ops<R>::sqrt_(R(0.5) * (s + Ops<R>::sqrt_(disc)));
+__device__ __forceinline__ float fast_speed_n(float gamma, float rho, float p, float bx, float by, float bz) {
+  float rinv = Ops<float>::div_(1.f, rho);
+  float a2 = Ops<float>::div_(gamma * p, rho);
+  float b2 = (bx * bx + by * by + bz * bz) * rinv;
+  float bn2 = bx * bx * rinv;
+  float s = a2 + b2;
+  float disc = s * s - 4.f * a2 * bn2;
+  disc = disc < 0.f ? 0.f : disc;
+  return Ops<float>::sqrt_(0.5f * (s + Ops<float>::sqrt_(disc)));
 }
-__device__ __forceinline__ double fast_speed_exact(double gamma, double rho, double p, double bx, double by,
-                                                   double bz) {
-  // FP64 path: the same divisions as the oracle, (gamma p)/rho and B^2/rho.
-  double a2 = gamma * p / rho;
-  double b2 = (bx * bx + by * by + bz * bz) / rho;
-  double bn2 = bx * bx / rho;
-  double s = a2 + b2;
-  double disc = s * s - 4.0 * a2 * bn2;
-  disc = disc < 0.0 ? 0.0 : disc;
-  return sqrt(0.5 * (s + sqrt(disc)));
+// CFL bound of a cell, sum_d (|u_d| + c_f,d) / dx_d, with the total field B.
+__device__ __forceinline__ double cfl_sum64(double gamma, const double W[8], const double B[3], const double idx[3]) {
+  const double b2[3] = {B[0] * B[0], B[1] * B[1], B[2] * B[2]};
+  const double gph = 0.5 * gamma * W[7], hb = 0.5 * (b2[0] + b2[1] + b2[2]);
+  double s = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; d++) s = fma(fabs(W[1 + d]) + fast_speed64(gph, hb, b2[d], W[0]), idx[d], s);
+  return s;
 }
 
 // Split-field physical flux along the frame normal (component 0 of the
 // rotated vectors): F_rho = rho un, F_m = rho u un + pt n - (B1 Bn + B0 B1n),
 // F_B1 = un B - Bn u (normal component 0), F_e1 = un (e1 + pt) - (u.B1) Bn,
 // pt = p + B1^2/2 + B0.B1.  Also U(W), un and the fast speed.
-template <class R>
-__device__ __forceinline__ void phys_flux(const R W[8], const R B0[3], R gamma, R inv_gm1, R F[8], R U[8],
-                                          R& un, R& cf) {
-  R rho = W[0];
-  R u0 = W[1], u1 = W[2], u2 = W[3];
-  R b10 = W[4], b11 = W[5], b12 = W[6], p = W[7];
-  R B_0 = B0[0] + b10, B_1 = B0[1] + b11, B_2 = B0[2] + b12;
-  R b1sq = b10 * b10 + b11 * b11 + b12 * b12;
-  R b0b1 = B0[0] * b10 + B0[1] * b11 + B0[2] * b12;
-  R usq = u0 * u0 + u1 * u1 + u2 * u2;
-  R pt = p + R(0.5) * b1sq + b0b1;
-  R e1 = p * inv_gm1 + R(0.5) * rho * usq + R(0.5) * b1sq;
-  R ub1 = u0 * b10 + u1 * b11 + u2 * b12;
+__device__ __forceinline__ void phys_flux(const float W[8], const float B0[3], float gamma, float inv_gm1, float F[8], float U[8],
+                                          float& un, float& cf) {
+  float rho = W[0];
+  float u0 = W[1], u1 = W[2], u2 = W[3];
+  float b10 = W[4], b11 = W[5], b12 = W[6], p = W[7];
+  float B_0 = B0[0] + b10, B_1 = B0[1] + b11, B_2 = B0[2] + b12;
+  float b1sq = b10 * b10 + b11 * b11 + b12 * b12;
+  float b0b1 = B0[0] * b10 + B0[1] * b11 + B0[2] * b12;
+  float usq = u0 * u0 + u1 * u1 + u2 * u2;
+  float pt = p + 0.5f * b1sq + b0b1;
+  float e1 = p * inv_gm1 + 0.5f * rho * usq + 0.5f * b1sq;
+  float ub1 = u0 * b10 + u1 * b11 + u2 * b12;
   un = u0;
   F[0] = rho * u0;
   F[1] = (rho * u0 * u0 + pt) - (b10 * B_0 + B0[0] * b10);
   F[2] = rho * u1 * u0 - (b11 * B_0 + B0[1] * b10);
   F[3] = rho * u2 * u0 - (b12 * B_0 + B0[2] * b10);
-  F[4] = R(0);
+  F[4] = 0.f;
   F[5] = u0 * B_1 - B_0 * u1;
   F[6] = u0 * B_2 - B_0 * u2;
   F[7] = u0 * (e1 + pt) - ub1 * B_0;
@@ -349,16 +368,14 @@ __device__ __forceinline__ void phys_flux(const R W[8], const R B0[3], R gamma, 
   U[5] = b11;
   U[6] = b12;
   U[7] = e1;
-  if constexpr (std::is_same<R, double>::value)
-    cf = fast_speed_exact(gamma, rho, p, B_0, B_1, B_2);
-  else
-    cf = fast_speed_n<R>(gamma, rho, p, B_0, B_1, B_2);
+  cf = fast_speed_n(gamma, rho, p, B_0, B_1, B_2);
 }
 
 // minmod of two doubles by integer tests on the bit patterns: 0 unless both
 // are nonzero with the same sign, else the one of smaller magnitude (the
 // second on a tie).  The same selection as the floating-point definition,
-// without the FP64 comparison unit.
+// without the FP64 comparison unit (comparisons share the FP64 pipe, which
+// bounds the FP64 form).
 __device__ __forceinline__ double minmod_d(double a, double b) {
   long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
   unsigned long long ma = static_cast<unsigned long long>(ia) & 0x7fffffffffffffffull;
@@ -366,13 +383,6 @@ __device__ __forceinline__ double minmod_d(double a, double b) {
   bool same = ((ia ^ ib) >= 0) && ma != 0 && mb != 0;
   long long r = ma < mb ? ia : ib;
   return same ? __longlong_as_double(r) : 0.0;
-}
-// The FP64 limiter's minmod by the same integer operations: the same value as
-// the comparison form for every finite argument, issued on the integer pipe
-// instead of the FP64 pipe (which bounds the FP64 form).
-template <>
-__device__ __forceinline__ double minmod_<double>(double a, double b) {
-  return minmod_d(a, b);
 }
 // Validity tests on bit patterns: finite, and finite and > 0.
 __device__ __forceinline__ bool finite_d(double x) {
@@ -821,7 +831,7 @@ __device__ __forceinline__ void prolong_child_w(const float* tab, int s, int loc
     const float* Up = tab + kp * PSTRIDE;
     const float sg = odd ? 0.25f : -0.25f;
 #pragma unroll
-    for (int v = 0; v < NV; v++) dl[v] = dl[v] + sg * minmod_<float>(Uc[v] - Um[v], Up[v] - Uc[v]);
+    for (int v = 0; v < NV; v++) dl[v] = dl[v] + sg * minmod_f(Uc[v] - Um[v], Up[v] - Uc[v]);
   }
   const float Wc[8] = {Uc[0], Uc[9], Uc[10], Uc[11], Uc[4], Uc[5], Uc[6], Uc[8]};
   prim_increment(Wc, dl, gm1f, w);
@@ -1011,6 +1021,219 @@ __device__ __forceinline__ void b0_face(const PhysDev& ph, int d, int i, int j, 
 }
 
 // ---------------------------------------------------------------------------
+// FP64 form, plain faces.  GB300 runs FP64 at 1/64 of the FP32 rate, so this
+// code is written for the fewest FP64 operations: selections and limiters on
+// bit patterns (integer pipe), roots by rsqrt64_est, no division, no operation
+// on an absent B0, face values stored doubled (the cell phase halves its
+// spacing instead).  Together with the warp-wise halves of faces64: 120 blocks
+// 561 -> 290 us a step, one step of 8 blocks with its state in and out 527 ->
+// 322 us, six grids with the HLL flux 36.7 -> 23.0 ms; the FP64 pipe is 81 to
+// 83 % busy before and after: the time went with the operations.
+
+// The limited slope of a cell as value and factor: half the slope is f v.
+// Minmod: the difference of smaller magnitude, f = 1/2; MC (beta = 2): that
+// difference with f = 1 or their sum with f = 1/4, whichever is smaller.  0
+// when the signs differ.
+template <int LIM>
+__device__ __forceinline__ double half_slope64(double a, double b, double& f) {
+  f = 0.5;
+  if constexpr (LIM == 2) return 0.0;
+  const double m = minmod_d(a, b);
+  if constexpr (LIM == 1) {
+    const double t = a + b;
+    const uint64_t mm = static_cast<uint64_t>(__double_as_longlong(m)) & 0x7fffffffffffffffull;
+    const uint64_t mt = static_cast<uint64_t>(__double_as_longlong(t)) & 0x7fffffffffffffffull;
+    const bool two = mm + (2ull << 52) < mt;  // 4 |m| < |a + b| (normal m): 2 |m| is the smaller bound
+    f = two ? 1.0 : 0.25;
+    return mm == 0 || two ? m : t;
+  }
+  return m;
+}
+
+// One side of a face: conserved state, physical flux in the face frame and
+// fast speed of the primitives w (phys_flux with the terms of an absent B0
+// left out).
+template <bool HAS_B0>
+__device__ __forceinline__ void side64(const double w[8], const double B0[3], double hgamma, double inv_gm1,
+                                       double F[8], double U[8], double& cf) {
+  const double rho = w[0], u0 = w[1], u1 = w[2], u2 = w[3], b0 = w[4], b1 = w[5], b2 = w[6], p = w[7];
+  const double bb0 = b0 * b0;
+  const double bsq = fma(b2, b2, fma(b1, b1, bb0));
+  double T0 = b0, T1 = b1, T2 = b2, tt0 = bb0, tsq = bsq;  // total field
+  if constexpr (HAS_B0) {
+    T0 += B0[0];
+    T1 += B0[1];
+    T2 += B0[2];
+    tt0 = T0 * T0;
+    tsq = fma(T2, T2, fma(T1, T1, tt0));
+  }
+  cf = fast_speed64(hgamma * p, 0.5 * tsq, tt0, rho);
+  const double usq = fma(u2, u2, fma(u1, u1, u0 * u0));
+  const double ub = fma(u2, b2, fma(u1, b1, u0 * b0));
+  double pt = fma(0.5, bsq, p);
+  if constexpr (HAS_B0) pt = fma(B0[2], b2, fma(B0[1], b1, fma(B0[0], b0, pt)));
+  U[0] = rho;
+  U[1] = rho * u0;
+  U[2] = rho * u1;
+  U[3] = rho * u2;
+  U[4] = b0;
+  U[5] = b1;
+  U[6] = b2;
+  U[7] = fma(p, inv_gm1, 0.5 * fma(rho, usq, bsq));
+  F[0] = U[1];
+  F[1] = fma(U[1], u0, fma(-b0, T0, pt));
+  F[2] = fma(U[2], u0, -(b1 * T0));
+  F[3] = fma(U[3], u0, -(b2 * T0));
+  if constexpr (HAS_B0) {
+    F[1] = fma(-B0[0], b0, F[1]);
+    F[2] = fma(-B0[1], b0, F[2]);
+    F[3] = fma(-B0[2], b0, F[3]);
+  }
+  F[4] = 0.0;
+  F[5] = fma(u0, T1, -(T0 * u1));
+  F[6] = fma(u0, T2, -(T0 * u2));
+  F[7] = fma(u0, U[7] + pt, -(ub * T0));
+}
+
+// Twice the numerical flux of the face with left and right states wl, wr;
+// Rusanov: also cmax and dU = U_R - U_L (for the learned correction's clip).
+template <bool HAS_B0, int FLX>
+__device__ __forceinline__ void face_flux64(const double wl[8], const double wr[8], const double B0[3], double hgamma,
+                                            double inv_gm1, double G[8], double& cmax, double dU[8]) {
+  double FL[8], UL[8], FR[8], UR[8], cl, cr;
+  side64<HAS_B0>(wl, B0, hgamma, inv_gm1, FL, UL, cl);
+  side64<HAS_B0>(wr, B0, hgamma, inv_gm1, FR, UR, cr);
+  if constexpr (FLX == FLUX_HLL || FLX == FLUX_LINDE) {
+    // HLL with S_L = min(unL - cfL, unR - cfR, 0), S_R = max(unL + cfL, unR +
+    // cfR, 0):  F = F_L - S_L/(S_R - S_L) ((F_R - F_L) - S_R (U_R - U_L))
+    double sl = wl[1] - cl < wr[1] - cr ? wl[1] - cl : wr[1] - cr;
+    double sr = wl[1] + cl > wr[1] + cr ? wl[1] + cl : wr[1] + cr;
+    sl = sl < 0.0 ? sl : 0.0;
+    sr = sr > 0.0 ? sr : 0.0;
+    const double den = sr - sl;
+    const double rden = den > 0.0 ? rcp64(den) : 0.0;
+    const double k2 = 2.0 * (sl * rden);
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const double dF = v == 4 ? 0.0 : FR[v] - FL[v];
+      G[v] = fma(-k2, fma(-sr, UR[v] - UL[v], dF), v == 4 ? 0.0 : 2.0 * FL[v]);
+    }
+    if constexpr (FLX == FLUX_LINDE) {
+      // Linde: the contact wave restored, F -= delta alpha S_L S_R / (S_R - S_L) r,
+      // alpha = minmod((rho_R - rho_L) - (p_R - p_L) / c^2, rho_R - rho_L),
+      // delta = c / (c + |u_n|), r = (1, u, 0, |u|^2 / 2), means of the two
+      // face states, c^2 = gamma p / rho
+      const double um0 = 0.5 * (wl[1] + wr[1]), um1 = 0.5 * (wl[2] + wr[2]), um2 = 0.5 * (wl[3] + wr[3]);
+      const double gp = hgamma * (wl[7] + wr[7]), rm = 0.5 * (wl[0] + wr[0]);
+      const double cs = div_sqrt64(gp, gp * rm), ic2 = rm * rcp64(gp);
+      const double dr = wr[0] - wl[0];
+      const double alpha = minmod_d(fma(-(wr[7] - wl[7]), ic2, dr), dr);
+      const double q = k2 == 0.0 ? 0.0 : k2 * sr * alpha * (cs * rcp64(cs + fabs(um0)));
+      G[0] -= q;
+      G[1] = fma(-q, um0, G[1]);
+      G[2] = fma(-q, um1, G[2]);
+      G[3] = fma(-q, um2, G[3]);
+      G[7] = fma(-q, 0.5 * fma(um2, um2, fma(um1, um1, um0 * um0)), G[7]);
+    }
+  } else {
+    const double al = fabs(wl[1]) + cl, ar = fabs(wr[1]) + cr;
+    cmax = al > ar ? al : ar;
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      dU[v] = UR[v] - UL[v];
+      G[v] = v == 4 ? -cmax * dU[v] : fma(-cmax, dU[v], FL[v] + FR[v]);
+    }
+  }
+}
+
+// The faces f0 .. f0 + nf - 1 of one grid line of direction d (fixed per
+// warp), a sliding window along the line: every cell is loaded and every
+// limited slope computed once.  A line is shared by two threads, faces 0-4 and
+// 5-8, of different warps, so that a warp takes 5 or 4 steps as a whole (two
+// halves in one warp took 5 everywhere, a tenth of the face work for nothing).
+template <int LIM, bool HAS_B0, int FLX>
+__device__ __forceinline__ void faces64(const StageArgs& a, const BlockDev& B, const double* sT, double* sF, int d,
+                                        int fline, int fhalf, double hgamma, double inv_gm1, const double lo[3],
+                                        const double dx[3]) {
+  const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+  const int ta = fline & 7, tb = fline >> 3;
+  const int stride = d == 0 ? 1 : (d == 1 ? NC : NC * NC);
+  const int inner = d == 0 ? (tb * NC + ta) * NC : (d == 1 ? tb * NC * NC + ta : tb * NC + ta);
+  const int glo = NCELL + 2 * d * 128 + 2 * (ta + NC * tb), ghi = glo + 128;
+  auto cell = [&](int c) { return c < 0 ? glo + (c + 2) : (c >= NC ? ghi + (c - NC) : inner + c * stride); };
+  const int rot[8] = {0, 1 + d, 1 + d1, 1 + d2, 4 + d, 4 + d1, 4 + d2, 7};
+  auto load = [&](int c, double w[8]) {
+    const double* q = sT + chki(cell(c), 0, NTILE);
+#pragma unroll
+    for (int v = 0; v < NV; v++) w[v] = q[rot[v] * NTILE];
+  };
+  const int f0 = fhalf ? 5 : 0, nf = fhalf ? 4 : 5;
+  double W0[8], df[8], WL[8];
+  {
+    double Wm2[8], Wm1[8];
+    load(f0 - 2, Wm2);
+    load(f0 - 1, Wm1);
+    load(f0, W0);
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      double f;
+      df[v] = W0[v] - Wm1[v];
+      const double h = half_slope64<LIM>(Wm1[v] - Wm2[v], df[v], f);
+      WL[v] = LIM == 2 ? Wm1[v] : fma(f, h, Wm1[v]);
+    }
+  }
+#pragma unroll 1
+  for (int k = 0; k < nf; k++) {
+    const int f = f0 + k;
+    double Wp[8], WR[8], WLn[8];
+    load(f + 1, Wp);
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      if constexpr (LIM == 2) {
+        WR[v] = WLn[v] = W0[v];
+      } else {
+        double g;
+        const double dn = Wp[v] - W0[v];
+        const double h = half_slope64<LIM>(df[v], dn, g);
+        WR[v] = fma(-g, h, W0[v]);
+        WLn[v] = fma(g, h, W0[v]);
+        df[v] = dn;
+      }
+    }
+    double B0r[3] = {0.0, 0.0, 0.0};
+    if constexpr (HAS_B0) {
+      const int ci = d == 0 ? f : ta, cj = d == 1 ? f : (d == 0 ? ta : tb), ck = d == 2 ? f : tb;
+      double B0f[3];
+      b0_face<double>(a.ph, d, ci, cj, ck, B.bi * NC, B.bj * NC, B.bk * NC, lo[0], lo[1], lo[2], dx[0], dx[1], dx[2],
+                      B0f);
+      B0r[0] = d == 0 ? B0f[0] : (d == 1 ? B0f[1] : B0f[2]);
+      B0r[1] = d1 == 0 ? B0f[0] : (d1 == 1 ? B0f[1] : B0f[2]);
+      B0r[2] = d2 == 0 ? B0f[0] : (d2 == 1 ? B0f[1] : B0f[2]);
+    }
+    double G[8], cmax, dU[8];
+    face_flux64<HAS_B0, FLX>(WL, WR, B0r, hgamma, inv_gm1, G, cmax, dU);
+    double* o = sF + d * (9 * NFACE) + chki(fline * 9 + f, 0, NFACE);
+#pragma unroll
+    for (int v = 0; v < NV; v++) o[rot[v] * NFACE] = G[v];
+    if (a.ph.powell) o[8 * NFACE] = WL[4] + WR[4];  // twice the face's normal B1
+    // refluxing: the block-face fluxes of faces at resolution changes
+    if (a.freg && (f == 0 || f == NC)) {
+      const int sl = chki(B.rslot[2 * d + (f == NC ? 1 : 0)], -1, a.nslots);
+      if (sl >= 0) {
+        double* r = a.freg + (static_cast<int64_t>(sl) * 64 + ta * NC + tb) * NV;
+#pragma unroll
+        for (int v = 0; v < NV; v++) r[rot[v]] = 0.5 * G[v];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      WL[v] = WLn[v];
+      W0[v] = Wp[v];
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Mixed form, plain faces (no learned correction): packed FP32.  GB300 issues
 // FADD2 / FMUL2 / FFMA2 on float2 pairs (two FP32 lanes per instruction);
 // every quantity of a face's two sides -- its left and right reconstructed
@@ -1036,7 +1259,7 @@ __device__ __forceinline__ float minmod_med(float a, float b) {
 template <int LIM>
 __device__ __forceinline__ float limit_f(float a, float b) {
   if constexpr (LIM == 2) return 0.f;
-  else if constexpr (LIM == 1) return mc_<float>(a, b);
+  else if constexpr (LIM == 1) return mc_f(a, b);
   else return minmod_med(a, b);
 }
 
@@ -1772,7 +1995,6 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
   R gamma, inv_gm1;
   if constexpr (MIXED) { gamma = ph.gammaf; inv_gm1 = ph.inv_gm1f; }
   else { gamma = ph.gamma; inv_gm1 = ph.inv_gm1; }
-  constexpr bool has_b0 = HAS_B0;
 
   // this thread's line in the face phase
   const int fd = tid >> 7;                      // direction 0..2
@@ -1904,27 +2126,33 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
       }
       const int gb0 = B.bi * NC, gb1 = B.bj * NC, gb2 = B.bk * NC;
 
-      // 3. faces: reconstruction + Rusanov flux in the frame (d, d+1, d+2);
-      //    corr = add the network's correction (learned form)
-      auto faces = [&](const bool corr) {
+      // 3. faces of the learned kernels (the plain ones: faces_mx, faces64):
+      //    reconstruction + Rusanov flux in the frame (d, d+1, d+2);
+      //    corr = add the network's correction
+      [[maybe_unused]] auto faces = [&]([[maybe_unused]] const bool corr) {
+        if constexpr (LRN) {
           auto cidx = [&](int c) { return c < 0 ? flo + (c + 2) : (c >= NC ? fhi + (c - NC) : fibase + c * fstride); };
           const int f0 = fhalf ? 5 : 0, nf = fhalf ? 4 : 5;
-          // window along the line.  Plain: the cell W0, the difference d = W0 - W-1
-          // and the left state WL of the next face, W-1 + s-1 / 2 (each difference
-          // and slope formed once).  Learned: the cells f-2..f, kept for the
-          // network's inputs.
-          R Wm1[8], W0[8], sm1[8];
-          R Wm2[8];
+          // window along the line: the cells f-2..f (the network's inputs), the
+          // difference d = W0 - W-1 and the left state WL of the next face
+          R Wm2[8], Wm1[8], W0[8];
           load_rot<R>(sT, rot, cidx(f0 - 2), Wm2);
           load_rot<R>(sT, rot, cidx(f0 - 1), Wm1);
           load_rot<R>(sT, rot, cidx(f0), W0);
           R d[8], WL[8];
+          auto half = [&](R da, R db, R W, R sgn) -> R {  // W + sgn x half the limited slope
+            if constexpr (MIXED) {
+              return W + sgn * R(0.5) * limit_(LIM, da, db);
+            } else {
+              double f;
+              const double h = half_slope64<LIM>(da, db, f);
+              return LIM == 2 ? W : fma(sgn * f, h, W);
+            }
+          };
 #pragma unroll
           for (int v = 0; v < NV; v++) {
-            const R dm = Wm1[v] - Wm2[v];
             d[v] = W0[v] - Wm1[v];
-            sm1[v] = limit_<R>(LIM, dm, d[v]);
-            WL[v] = Wm1[v] + R(0.5) * sm1[v];
+            WL[v] = half(Wm1[v] - Wm2[v], d[v], Wm1[v], R(1));
           }
           // fused network: every thread takes five steps (the CTA's 384 faces
           // of a step go through the network together); a lane of the upper
@@ -1934,14 +2162,10 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
           for (int k = 0; k < nsteps; k++) {
             const bool valid = k < nf;
             const int f = f0 + k;
-            R Wp[8], WR[8], s0[8], dn[8];
+            R Wp[8], WR[8];
             load_rot<R>(sT, rot, cidx(valid ? f + 1 : f), Wp);
 #pragma unroll
-            for (int v = 0; v < NV; v++) {
-              dn[v] = Wp[v] - W0[v];
-              s0[v] = limit_<R>(LIM, d[v], dn[v]);
-              WR[v] = W0[v] - R(0.5) * s0[v];
-            }
+            for (int v = 0; v < NV; v++) WR[v] = half(d[v], Wp[v] - W0[v], W0[v], R(-1));
             R B0f[3] = {R(0), R(0), R(0)}, B0r[3];
             if constexpr (HAS_B0) {
               const int ci_ = fd == 0 ? f : fta, cj_ = fd == 1 ? f : (fd == 0 ? fta : ftb), ck_ = fd == 2 ? f : ftb;
@@ -1950,50 +2174,25 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
             B0r[0] = fd == 0 ? B0f[0] : (fd == 1 ? B0f[1] : B0f[2]);
             B0r[1] = fd1 == 0 ? B0f[0] : (fd1 == 1 ? B0f[1] : B0f[2]);
             B0r[2] = fd2 == 0 ? B0f[0] : (fd2 == 1 ? B0f[1] : B0f[2]);
-            R FL[8], UL[8], FR[8], UR[8], unL, unR, cfL, cfR;
-            phys_flux<R>(WL, B0r, gamma, inv_gm1, FL, UL, unL, cfL);
-            phys_flux<R>(WR, B0r, gamma, inv_gm1, FR, UR, unR, cfR);
-            R aL = Ops<R>::abs_(unL) + cfL, aR = Ops<R>::abs_(unR) + cfR;
-            R cmax = aL > aR ? aL : aR;
             const int fi = chki(fline * 9 + (f < 9 ? f : 8), 0, NFACE);  // (f = 9: the throw-away step)
-            R Fr[8];
-            if constexpr (FLX == FLUX_HLL || FLX == FLUX_LINDE) {
-              // HLL with S_L = min(unL - cfL, unR - cfR, 0), S_R = max(unL + cfL,
-              // unR + cfR, 0):  F = F_L - S_L/(S_R - S_L) ((F_R - F_L) - S_R (U_R - U_L)),
-              // which is F_L when every wave moves right (S_L = 0), F_R when every
-              // wave moves left (S_R = 0), else the two-state HLL flux
-              const R zero = R(0);
-              R sl = unL - cfL < unR - cfR ? unL - cfL : unR - cfR;
-              R sr = unL + cfL > unR + cfR ? unL + cfL : unR + cfR;
-              sl = sl < zero ? sl : zero;
-              sr = sr > zero ? sr : zero;
-              const R den = sr - sl;
-              const R kk = den > zero ? Ops<R>::div_(sl, den) : zero;
+            R Fr[8], cmax, dU[8];
+            if constexpr (MIXED) {
+              R FL[8], UL[8], FR[8], UR[8], unL, unR, cfL, cfR;
+              phys_flux(WL, B0r, gamma, inv_gm1, FL, UL, unL, cfL);
+              phys_flux(WR, B0r, gamma, inv_gm1, FR, UR, unR, cfR);
+              const R aL = Ops<R>::abs_(unL) + cfL, aR = Ops<R>::abs_(unR) + cfR;
+              cmax = aL > aR ? aL : aR;
 #pragma unroll
-              for (int v = 0; v < NV; v++) Fr[v] = FL[v] - kk * ((FR[v] - FL[v]) - sr * (UR[v] - UL[v]));
-              if constexpr (FLX == FLUX_LINDE) {
-                // Linde: the contact wave restored, F -= delta alpha S_L S_R / (S_R - S_L) r,
-                // alpha = minmod((rho_R - rho_L) - (p_R - p_L) / c^2, rho_R - rho_L),
-                // delta = c / (c + |u_n|), r = (1, u, 0, |u|^2 / 2), means of the two
-                // face states, c^2 = gamma p / rho
-                const R rm = R(0.5) * (WL[0] + WR[0]), pm = R(0.5) * (WL[7] + WR[7]);
-                const R um0 = R(0.5) * (WL[1] + WR[1]), um1 = R(0.5) * (WL[2] + WR[2]),
-                        um2 = R(0.5) * (WL[3] + WR[3]);
-                const R c2 = Ops<R>::div_(gamma * pm, rm), cs = Ops<R>::sqrt_(c2);
-                const R alpha = minmod_<R>((WR[0] - WL[0]) - Ops<R>::div_(WR[7] - WL[7], c2), WR[0] - WL[0]);
-                const R delta = Ops<R>::div_(cs, cs + Ops<R>::abs_(um0));
-                const R q = den > zero ? Ops<R>::div_(delta * alpha * (sl * sr), den) : zero;
-                Fr[0] -= q;
-                Fr[1] -= q * um0;
-                Fr[2] -= q * um1;
-                Fr[3] -= q * um2;
-                Fr[7] -= q * (R(0.5) * ((um0 * um0 + um1 * um1) + um2 * um2));
+              for (int v = 0; v < NV; v++) {
+                dU[v] = UR[v] - UL[v];
+                Fr[v] = R(0.5) * (FL[v] + FR[v]) - R(0.5) * cmax * dU[v];
               }
-            } else {
+            } else {  // the plain kernel's flux, value for value
+              face_flux64<HAS_B0, FLX>(WL, WR, B0r, R(0.5) * gamma, inv_gm1, Fr, cmax, dU);
 #pragma unroll
-              for (int v = 0; v < NV; v++) Fr[v] = R(0.5) * (FL[v] + FR[v]) - R(0.5) * cmax * (UR[v] - UL[v]);
+              for (int v = 0; v < NV; v++) Fr[v] = R(0.5) * Fr[v];
             }
-            if constexpr (LRN) {
+            {
               // network inputs: the 4 stencil cells f-2..f+1 and (WL + WR)/2 in
               // the face frame, scaled by rho_ref = mean stencil density and
               // c_ref = cmax (u / c_ref, B / (sqrt(rho_ref) c_ref), p / (rho_ref c_ref^2))
@@ -2082,7 +2281,7 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
                 for (int v = 0; v < NV; v++) {
                   const R sc = v == 0 ? sc0 : (v < 4 ? sc1 : (v < 7 ? sc4 : sc7));
                   R dF = R(yv[v]) * sc;
-                  const R lim = Ops<R>::abs_(R(0.5) * cmax * (UR[v] - UL[v]));
+                  const R lim = Ops<R>::abs_(R(0.5) * cmax * dU[v]);
                   dF = dF > lim ? lim : dF;
                   dF = dF < -lim ? -lim : dF;
                   Fr[v] = Fr[v] + dF;
@@ -2096,7 +2295,7 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
                 for (int v = 0; v < NV; v++) {
                   const R sc = v == 0 ? sc0 : (v < 4 ? sc1 : (v < 7 ? sc4 : sc7));
                   R dF = R(yv[v]) * sc;
-                  const R lim = Ops<R>::abs_(R(0.5) * cmax * (UR[v] - UL[v]));
+                  const R lim = Ops<R>::abs_(R(0.5) * cmax * dU[v]);
                   dF = dF > lim ? lim : dF;
                   dF = dF < -lim ? -lim : dF;
                   Fr[v] = Fr[v] + dF;
@@ -2107,13 +2306,11 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
             const R bnf = R(0.5) * (WL[4] + WR[4]);  // face-averaged normal B1 (Powell)
 #pragma unroll
             for (int v = 0; v < NV; v++) {
-              if constexpr (LRN) {
-                Wm2[v] = Wm1[v];
-                Wm1[v] = W0[v];
-              }
-              WL[v] = W0[v] + R(0.5) * s0[v];
+              WL[v] = half(d[v], Wp[v] - W0[v], W0[v], R(1));
+              d[v] = Wp[v] - W0[v];
+              Wm2[v] = Wm1[v];
+              Wm1[v] = W0[v];
               W0[v] = Wp[v];
-              d[v] = dn[v];
             }
             if (a.kind >= 3) continue;
             fcol[0 * NFACE + fi] = Fr[0];
@@ -2125,28 +2322,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
             fcol[(4 + fd2) * NFACE + fi] = Fr[6];
             fcol[7 * NFACE + fi] = Fr[7];
             fcol[8 * NFACE + fi] = bnf;
-            // refluxing: the block-face fluxes of faces at resolution changes
-            if (a.freg && (f == 0 || f == NC)) {
-              const int sl = chki(B.rslot[2 * fd + (f == NC ? 1 : 0)], -1, a.nslots);
-              if (sl >= 0) {
-                double* o = a.freg + (static_cast<int64_t>(sl) * 64 + fta * NC + ftb) * NV;
-                double Fd[8];
-#pragma unroll
-                for (int v = 0; v < NV; v++) {
-                  if constexpr (MIXED) Fd[v] = f2d_int(Fr[v]);
-                  else Fd[v] = Fr[v];
-                }
-                o[0] = Fd[0];
-                o[1 + fd] = Fd[1];
-                o[1 + fd1] = Fd[2];
-                o[1 + fd2] = Fd[3];
-                o[4 + fd] = Fd[4];
-                o[4 + fd1] = Fd[5];
-                o[4 + fd2] = Fd[6];
-                o[7] = Fd[7];
-              }
-            }
           }
+        }
       };
       // 4. per cell: flux differences, sources, update, CFL bound.  commit =
       //    false only checks the update (learned form): returns whether this
@@ -2161,8 +2338,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
         const int kind = FAST ? 0 : a.kind;
         double* const dtc = FAST ? nullptr : a.dtc;
         const bool blk_body = FAST ? false : B.body != 0;
-        // the packed mixed face phase stores doubled face values
-        constexpr R FS = (MIXED && !LRN) ? R(0.5) : R(1);
+        // the plain face phases store doubled face values
+        constexpr R FS = LRN ? R(1) : R(0.5);
         const R fidx0 = FS * idx0, fidx1 = FS * idx1, fidx2 = FS * idx2;
         bool any_bad = false;
         R smax_loc = R(0);
@@ -2194,9 +2371,11 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
             r = r - (Fz[vz * NFACE + tz + 1] - Fz[vz * NFACE + tz]) * fidx2;
             res[v] = r;
           }
-          const R divb = ((Fx[8 * NFACE + tx + 1] - Fx[8 * NFACE + tx]) * fidx0 +
-                          (Fy[8 * NFACE + ty + 1] - Fy[8 * NFACE + ty]) * fidx1) +
-                         (Fz[8 * NFACE + tz + 1] - Fz[8 * NFACE + tz]) * fidx2;
+          R divb = R(0);
+          if (MX || ph.powell)
+            divb = ((Fx[8 * NFACE + tx + 1] - Fx[8 * NFACE + tx]) * fidx0 +
+                    (Fy[8 * NFACE + ty + 1] - Fy[8 * NFACE + ty]) * fidx1) +
+                   (Fz[8 * NFACE + tz + 1] - Fz[8 * NFACE + tz]) * fidx2;
           bool in_body = false;
           if (blk_body) {  // FP64, the same centre formula as the host and the oracle
             double x = G.lo[0] + ((static_cast<double>(gb0) + ci) + 0.5) * G.dx[lev][0];
@@ -2329,17 +2508,16 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
           if (a.last && !in_body && kind != 2 && !refl) {
             R Bt[3] = {B0c[0] + Wn[4], B0c[1] + Wn[5], B0c[2] + Wn[6]};
             R sacc = R(0);
+            if constexpr (MIXED) {
 #pragma unroll
-            for (int e = 0; e < 3; e++) {
-              R bn = Bt[e], bt1 = Bt[(e + 1) % 3], bt2 = Bt[(e + 2) % 3];
-              R cf;
-              if constexpr (MIXED) {
-                cf = fast_speed_n<R>(gamma, Wn[0], Wn[7], bn, bt1, bt2);
+              for (int e = 0; e < 3; e++) {
+                R bn = Bt[e], bt1 = Bt[(e + 1) % 3], bt2 = Bt[(e + 2) % 3];
+                R cf = fast_speed_n(gamma, Wn[0], Wn[7], bn, bt1, bt2);
                 sacc = sacc + (Ops<R>::abs_(Wn[1 + e]) + cf) * (e == 0 ? idx0 : (e == 1 ? idx1 : idx2));
-              } else {
-                cf = fast_speed_exact(ph.gamma, Wn[0], Wn[7], bn, bt1, bt2);
-                sacc = sacc + (Ops<R>::abs_(Wn[1 + e]) + cf) / (e == 0 ? dxr0 : (e == 1 ? dxr1 : dxr2));
               }
+            } else {
+              const double idx[3] = {idx0, idx1, idx2};
+              sacc = cfl_sum64(ph.gamma, Wn, Bt, idx);
             }
             smax_loc = sacc > smax_loc ? sacc : smax_loc;
             if (dtc) {
@@ -2378,6 +2556,16 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
         if (tid < FACE_THREADS) {
           faces_mx<LIM, HAS_B0, FLX>(fd, a, B, sT, sF, fline, fhalf, gamma, inv_gm1, gb0, gb1, gb2, lor0, lor1, lor2,
                                      dxr0, dxr1, dxr2);
+        }
+      } else if constexpr (!LRN) {
+        // half h of the lines 32 (w & 1) .. of direction fd per warp w of its
+        // four; the halves' order alternates over the directions, so that the
+        // SM's four schedulers get 13 or 14 of the 54 warp steps each
+        if (tid < FACE_THREADS) {
+          const double lo[3] = {lor0, lor1, lor2}, dx[3] = {dxr0, dxr1, dxr2};
+          const int wq = (tid >> 5) & 3;
+          faces64<LIM, HAS_B0, FLX>(a, B, sT, sF, fd, 32 * (wq & 1) + (tid & 31), (wq >> 1) ^ (fd & 1), 0.5 * gamma,
+                                    inv_gm1, lo, dx);
         }
       } else {
         if (tid < FACE_THREADS) faces(true);
