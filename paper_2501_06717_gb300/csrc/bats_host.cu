@@ -346,6 +346,13 @@ int build_grid(bats_t* h, const bats_grid_desc& d, int gidx, int block0, std::ve
     }
   }
   for (int a = 0; a < 3; a++) gd.lof[a] = static_cast<float>(d.lo[a]);
+  for (int b = 0; b < d.n_leaves; b++) {
+    BlockDev& B = blocks[block0 + b];
+    for (int a = 0; a < 3; a++) {
+      B.idxf[a] = gd.idxf[B.level][a];
+      B.dxf[a] = gd.dxf[B.level][a];
+    }
+  }
   // blocks with a cell centre inside the body (same FP64 centre formula as the kernels)
   if (d.body_r > 0.0) {
     for (int b = 0; b < d.n_leaves; b++) {
@@ -473,7 +480,13 @@ int launch_stage_one(bats_t* h, const StageArgs& a0, bool make_ghosts = true, bo
   }
   int nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
   int grid = nitems;
-  if (one_per_sm) {
+  if (one_per_sm || (mixed && !a.learned && a.kind < 3)) {
+    // the plain mixed kernel overlaps a CTA's successive blocks, so its CTAs
+    // (one per SM) always walk over the items; at least eight items per CTA, so
+    // that the last round costs at most an eighth (6,084 blocks on 152 SMs: 16.5
+    // ms per 40 steps in items of 8 blocks, 15.7 ms in single blocks)
+    if (!a.learned) a.blocks_per_item = std::max(1, std::min(a.blocks_per_item, a.nblocks / (8 * h->num_sms)));
+    nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
     grid = std::min(nitems, h->num_sms);
   } else if (h->persistent) {
     int per_sm = h->ctas_per_sm > 0 ? std::min(h->ctas_per_sm, h->occ[mixed]) : h->occ[mixed];
@@ -730,11 +743,12 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// The four tensor maps of an FP32 state buffer W (block-major [block][8][512])
-// viewed as the 4-D tensor (i, j, k, 8 * block + v): the interior box
-// 8 x 8 x 8 x 8 with the 32-byte swizzle, and the face-slab boxes of the
-// neighbour's cells nearest a face, 4 x 8 x 8 x 8 (x; a TMA box row is at
-// least 16 bytes), 8 x 2 x 8 x 8 (y) and 8 x 8 x 2 x 8 (z).
+// The four tensor maps of an FP32 state buffer W (block-major [block][8][512]):
+// the interior as the 4-D tensor (32 cells: four rows of i, j / 4, k,
+// 8 * block + v), box 32 x 2 x 8 x 8 with the 128-byte swizzle; and, of the
+// 4-D tensor (i, j, k, 8 * block + v), the face-slab boxes of the neighbour's
+// cells nearest a face, 4 x 8 x 8 x 8 (x; a TMA box row is at least 16 bytes),
+// 8 x 2 x 8 x 8 (y) and 8 x 8 x 2 x 8 (z).
 static int encode_tile_maps(bats_t* h, float* W, CUtensorMap tm[4]) {
   static EncodeTiledFn encode = nullptr;
   if (!encode) {
@@ -748,10 +762,13 @@ static int encode_tile_maps(bats_t* h, float* W, CUtensorMap tm[4]) {
   const cuuint64_t dims[4] = {NC, NC, NC, static_cast<cuuint64_t>(h->nbt) * NV};
   const cuuint64_t strides[3] = {NC * sizeof(float), NC * NC * sizeof(float), NCELL * sizeof(float)};
   const cuuint32_t estr[4] = {1, 1, 1, 1};
-  const cuuint32_t boxes[4][4] = {{NC, NC, NC, NV}, {4, NC, NC, NV}, {NC, 2, NC, NV}, {NC, NC, 2, NV}};
+  const cuuint64_t idims[4] = {32, 2, NC, static_cast<cuuint64_t>(h->nbt) * NV};
+  const cuuint64_t istrides[3] = {32 * sizeof(float), NC * NC * sizeof(float), NCELL * sizeof(float)};
+  const cuuint32_t boxes[4][4] = {{32, 2, NC, NV}, {4, NC, NC, NV}, {NC, 2, NC, NV}, {NC, NC, 2, NV}};
   for (int m = 0; m < 4; m++) {
-    CUresult r = encode(&tm[m], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, W, dims, strides, boxes[m], estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, m == 0 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE,
+    CUresult r = encode(&tm[m], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, W, m ? dims : idims, m ? strides : istrides,
+                        boxes[m], estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                        m == 0 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(h, BATS_ERR_CUDA, "cuTensorMapEncodeTiled failed for a state buffer");
   }

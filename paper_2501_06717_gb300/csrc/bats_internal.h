@@ -18,16 +18,15 @@ constexpr int NGHOST = 768;    // face-slab ghost cells (6 x 2 x 64)
 constexpr int NTILE = 1280;    // interior + face-slab ghosts
 constexpr int MAXLEV = 14;
 constexpr int FACE_THREADS = 384;   // face phase: two threads per grid line, three directions
-// stage CTA threads per form: 384 both (2 CTAs per SM at 80 registers in the
-// mixed form, 1 at 168 in FP64).  512 threads (one per cell in the cell phase)
-// measured slower in the mixed form: 64 registers spill in the face phase.
-constexpr int STAGE_THREADS_MIXED = 384, STAGE_THREADS_FP64 = 384;
+constexpr int STAGE_THREADS = 384;  // CTA of the FP64 and the learned stage kernels (1 per SM)
+// CTA of the mixed plain stage kernel (1 per SM, 80 registers): 12 warps for the
+// faces, 12 for the cells
+constexpr int MX_FACE_WARPS = 12, MX_CELL_WARPS = 12, MX_THREADS = 32 * (MX_FACE_WARPS + MX_CELL_WARPS);
 
 // Mixed-form tile of the plain stage kernel (FP32 primitives, floats):
-//  * interior [8 v][8 k][8 j][8 i] in the 32-byte TMA swizzle: the two
-//    16-byte halves of each 8-cell row are exchanged in rows with j >= 4, so
-//    that cell (i, j, k) of variable v sits at
-//    v * 512 + 64 k + 8 j + (i ^ (4 * ((j >> 2) & 1)));
+//  * interior [8 v][8 k][8 j][8 i] in the 128-byte TMA swizzle (the 16-byte
+//    chunk index within each 128 bytes XORed with the 128-byte row's number mod
+//    8): cell c = 64 k + 8 j + i of a variable sits at c ^ (((c >> 5) & 7) << 2);
 //  * the six face slabs in the layouts that tensor copies of the neighbour's
 //    cells nearest the face produce, in the neighbour's own cell order:
 //    -x / +x [8 v][8 k][8 j][4 i] (the neighbour's cells 4-7 / 0-3 along x:
@@ -59,15 +58,17 @@ struct GridDev {
   float lof[3];
 };
 
-struct BlockDev {
+struct alignas(16) BlockDev {     // 128 bytes: the mixed plain kernel stages it by a bulk copy
   int32_t grid, level, bi, bj, bk;
   int32_t ftype[6];              // FaceType per face (-x, +x, -y, +y, -z, +z)
   int32_t fnb[6];                // neighbour block (global index) for SAME / COARSER
   int32_t amr;                   // 1 if any face is COARSER or FINER
   int32_t body;                  // 1 if some cell centre lies inside the inner body
   int32_t rslot[6];              // refluxing: flux-register slot of a COARSER/FINER face, else -1
-  int32_t pad_[2];
+  float idxf[3], dxf[3];         // 1/dx and dx of the block's level (FP32)
+  int32_t pad_;
 };
+static_assert(sizeof(BlockDev) == 128, "one bulk copy per block record");
 
 struct PhysDev {
   double gamma, gm1, inv_gm1;

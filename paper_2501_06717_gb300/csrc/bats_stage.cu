@@ -465,13 +465,18 @@ constexpr size_t kDebugFillMxSmem = sizeof(float) * MX_TILE + 1024;
 __global__ void k_debug_fill_mx(const __grid_constant__ StageArgs a, int b0, int nb, double* T) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t bar;
+  __shared__ BlockDev rec;
   const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
   float* sT = reinterpret_cast<float*>(smem_raw + pad);
   const int blk = b0 + blockIdx.x;
   if (threadIdx.x == 0) mbar_init(&bar, 1);
   __syncthreads();
-  mx_stage_tile(a, a.blocks[blk], blk, sT, &bar, threadIdx.x, blockDim.x);
+  const MxPlan plan = mx_plan(a, blk);
+  const unsigned fill = mx_fill_mask(a, plan);
+  if (threadIdx.x == 0) mx_issue_copies(a, plan, fill, blk, sT, &rec, &bar);
   if (!mbar_wait_bounded(&bar, 0, a.err)) mbar_wait_bounded(&bar, 0, a.err);
+  __syncthreads();
+  mx_fill_slabs(a, a.blocks[blk], fill, sT, threadIdx.x, blockDim.x);
   __syncthreads();
   const int tile = 12 * 12 * 12;
   for (int e = threadIdx.x; e < tile; e += blockDim.x) {
@@ -479,7 +484,7 @@ __global__ void k_debug_fill_mx(const __grid_constant__ StageArgs a, int b0, int
     const int oi = (i < 0 || i >= NC), oj = (j < 0 || j >= NC), ok = (k < 0 || k >= NC);
     int t = -1, vs = 0;
     if (oi + oj + ok == 0) {
-      t = mx_int(i, j, k);
+      t = mx_int((k * NC + j) * NC + i);
       vs = NCELL;
     } else if (oi + oj + ok == 1) {
       const int d = oi ? 0 : (oj ? 1 : 2);
@@ -517,9 +522,15 @@ static size_t stage_smem(bool mixed, bool lrn) {
 using StageFn = void (*)(const StageArgs);
 template <bool MIXED, bool LRN, int FLX>
 StageFn stage_fn_l(int lim, bool b0) {
-  if (lim == 2) return b0 ? k_stage<MIXED, 2, true, LRN, FLX> : k_stage<MIXED, 2, false, LRN, FLX>;
-  if (lim == 1) return b0 ? k_stage<MIXED, 1, true, LRN, FLX> : k_stage<MIXED, 1, false, LRN, FLX>;
-  return b0 ? k_stage<MIXED, 0, true, LRN, FLX> : k_stage<MIXED, 0, false, LRN, FLX>;
+  if constexpr (MIXED && !LRN) {
+    if (lim == 2) return b0 ? k_stage_mx<2, true, FLX> : k_stage_mx<2, false, FLX>;
+    if (lim == 1) return b0 ? k_stage_mx<1, true, FLX> : k_stage_mx<1, false, FLX>;
+    return b0 ? k_stage_mx<0, true, FLX> : k_stage_mx<0, false, FLX>;
+  } else {
+    if (lim == 2) return b0 ? k_stage<MIXED, 2, true, LRN, FLX> : k_stage<MIXED, 2, false, LRN, FLX>;
+    if (lim == 1) return b0 ? k_stage<MIXED, 1, true, LRN, FLX> : k_stage<MIXED, 1, false, LRN, FLX>;
+    return b0 ? k_stage<MIXED, 0, true, LRN, FLX> : k_stage<MIXED, 0, false, LRN, FLX>;
+  }
 }
 // The learned correction is defined on the Rusanov flux only (the host rejects
 // learned + HLL or Linde), so the other fluxes are instantiated for the plain
@@ -556,10 +567,10 @@ cudaError_t stage_setup(int occ[2]) {
     e = cudaFuncSetAttribute(k_debug_fill_mx, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(kDebugFillMxSmem));
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], stage_fn<false>(0, false), StageCfg<false>::THREADS,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[0], stage_fn<false>(0, false), STAGE_THREADS,
                                                       StageCfg<false>::SMEM);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], stage_fn<true>(0, false), StageCfg<true>::THREADS,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ[1], stage_fn<true>(0, false), MX_THREADS,
                                                       stage_smem(true, false));
   return e;
 }
@@ -569,9 +580,9 @@ cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const Sta
   const bool lrn = a.learned || a.kind >= 3;
   const int flux = a.ph.flux;
   if (mixed)
-    stage_fn<true>(a.ph.limiter, b0, lrn, flux)<<<grid, StageCfg<true>::THREADS, stage_smem(true, lrn), st>>>(a);
+    stage_fn<true>(a.ph.limiter, b0, lrn, flux)<<<grid, lrn ? STAGE_THREADS : MX_THREADS, stage_smem(true, lrn), st>>>(a);
   else
-    stage_fn<false>(a.ph.limiter, b0, lrn, flux)<<<grid, StageCfg<false>::THREADS, StageCfg<false>::SMEM, st>>>(a);
+    stage_fn<false>(a.ph.limiter, b0, lrn, flux)<<<grid, STAGE_THREADS, StageCfg<false>::SMEM, st>>>(a);
   return cudaGetLastError();
 }
 

@@ -9,9 +9,15 @@ namespace batsk {
 using StageFn = void (*)(const StageArgs);
 template <bool MIXED, int FLX>
 static StageFn pick(int lim, bool b0) {
-  if (lim == 2) return b0 ? k_stage<MIXED, 2, true, false, FLX> : k_stage<MIXED, 2, false, false, FLX>;
-  if (lim == 1) return b0 ? k_stage<MIXED, 1, true, false, FLX> : k_stage<MIXED, 1, false, false, FLX>;
-  return b0 ? k_stage<MIXED, 0, true, false, FLX> : k_stage<MIXED, 0, false, false, FLX>;
+  if constexpr (MIXED) {
+    if (lim == 2) return b0 ? k_stage_mx<2, true, FLX> : k_stage_mx<2, false, FLX>;
+    if (lim == 1) return b0 ? k_stage_mx<1, true, FLX> : k_stage_mx<1, false, FLX>;
+    return b0 ? k_stage_mx<0, true, FLX> : k_stage_mx<0, false, FLX>;
+  } else {
+    if (lim == 2) return b0 ? k_stage<false, 2, true, false, FLX> : k_stage<false, 2, false, false, FLX>;
+    if (lim == 1) return b0 ? k_stage<false, 1, true, false, FLX> : k_stage<false, 1, false, false, FLX>;
+    return b0 ? k_stage<false, 0, true, false, FLX> : k_stage<false, 0, false, false, FLX>;
+  }
 }
 StageFn stage_fn_flux(bool mixed, int lim, bool b0, int flux) {
   if (flux == FLUX_LINDE) return mixed ? pick<true, FLUX_LINDE>(lim, b0) : pick<false, FLUX_LINDE>(lim, b0);

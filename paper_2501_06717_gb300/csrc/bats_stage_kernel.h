@@ -58,6 +58,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
@@ -78,6 +81,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// A load that stays where it is written (ahead of a barrier).
+__device__ __forceinline__ double ld_early(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
 // Hint that [p, p + bytes) will be read soon: bring it into L2 (p 16-byte
 // aligned, bytes a multiple of 16).
 __device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
@@ -92,9 +101,9 @@ __device__ __forceinline__ uint64_t globaltimer() {
 // Wait for an mbarrier phase; gives up after ~1 s of wall time, records
 // ERR_TIMEOUT and returns false (the caller then waits once more, bounded,
 // so that no bulk copy is left in flight into this CTA's shared memory).
-static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int32_t* err) {
+__device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity, int32_t* err) {
   if (mbar_try_wait(bar, parity)) return true;
-  uint64_t t0 = globaltimer();
+  const uint64_t t0 = globaltimer();
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
     if (globaltimer() - t0 > 1000000000ull) {
@@ -102,6 +111,9 @@ static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t pa
       return false;
     }
   }
+}
+static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int32_t* err) {
+  return mbar_wait_inline(bar, parity, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -847,8 +859,8 @@ __device__ __forceinline__ int tile_index(int d, int c, int a, int b) {
 }
 
 // Staged tile of the mixed plain kernel (layouts: MX_* in bats_internal.h).
-// Interior cell (i, j, k) of one variable in the swizzled tile.
-__device__ __forceinline__ int mx_int(int i, int j, int k) { return 64 * k + 8 * j + (i ^ (4 * ((j >> 2) & 1))); }
+// Interior cell c = 64 k + 8 j + i of one variable in the swizzled tile.
+__device__ __forceinline__ int mx_int(int c) { return c ^ (((c >> 5) & 7) << 2); }
 // Start of face s's slab, the variable stride in it, and the element of
 // ghost cell c (-2, -1 or 8, 9 along the face's axis) at transverse
 // coordinates (ta, tb) (increasing axis order).
@@ -991,12 +1003,11 @@ __device__ __forceinline__ void fill_ghosts_block_mixed(const StageArgs& a, cons
 template <bool MIXED>
 struct StageCfg {
   using R = typename std::conditional<MIXED, float, double>::type;
-  static constexpr int THREADS = MIXED ? STAGE_THREADS_MIXED : STAGE_THREADS_FP64;
   static constexpr int NFC = 9;  // per face: 8 fluxes and the face-averaged normal B1
   static constexpr size_t SMEM = sizeof(R) * (NV * NTILE + 3 * NFC * NFACE);
-  // the mixed plain kernel's staged tile (MX_TILE floats, 1024-byte aligned
-  // for the swizzled tensor copy) and its face values
-  static constexpr size_t SMEM_MX = sizeof(float) * (MX_TILE + 3 * NFC * NFACE) + 1024;
+  // the mixed plain kernel: two staged tiles (MX_TILE floats, 1024-byte
+  // aligned for the swizzled tensor copy) and two sets of face values
+  static constexpr size_t SMEM_MX = sizeof(float) * 2 * (MX_TILE + 3 * NFC * NFACE) + 1024;
 };
 
 // Load the 8 primitives of tile cell `idx` in the face frame (normal, t1, t2):
@@ -1368,7 +1379,7 @@ __device__ __forceinline__ void face_flux2(const float2 W2[8], const float B0r[3
 // ---------------------------------------------------------------------------
 // Mixed form, plain stage kernel: tile staging.  Per block one thread issues
 // the copies that complete on the block's mbarrier: the interior by one
-// tensor copy (box 8 x 8 x 8 cells x 8 variables, 32-byte swizzle), each
+// tensor copy (8 x 8 x 8 cells x 8 variables, 128-byte swizzle), each
 // same-level face slab by one tensor copy of the neighbour's cells nearest
 // the face (stage_tma = 1), and each precomputed slab of a face at a
 // resolution change by a bulk copy from the ghost-slab buffer.  The threads
@@ -1387,80 +1398,66 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, in
 }
 
 
-// Primitives of face-slab ghost (s, layer, ta, tb) of block blk for a
-// same-level, outflow or inflow face: the neighbour's (or, outflow, the
-// block's own boundary) cell from Win, or the inflow state.
-__device__ __forceinline__ void mx_ghost_value(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk,
-                                               int s, int layer, int ta, int tb, float w[8]) {
-  const int d = s >> 1, side = s & 1;
-  const int ft = B.ftype[s];
-  if (ft == FACE_INFLOW) {
-#pragma unroll
-    for (int v = 0; v < NV; v++) w[v] = G.Winflow32[v];
-    return;
-  }
-  const int c = side ? NC + layer : layer - 2;
-  const int src = chki(ft == FACE_SAME ? B.fnb[s] : blk, 0, a.nblocks);
-  const int cn = ft == FACE_SAME ? (side ? c - NC : c + NC) : (side ? NC - 1 : 0);
-  const int i = d == 0 ? cn : ta, j = d == 1 ? cn : (d == 0 ? ta : tb), k = d == 2 ? cn : tb;
-  const float* p = a.Win + static_cast<int64_t>(src) * (NV * NCELL) + chki((k * NC + j) * NC + i, 0, NCELL);
-#pragma unroll
-  for (int v = 0; v < NV; v++) w[v] = p[v * NCELL];
-}
-
-// Faces of block B whose slabs come by copies: tensor copies (same level,
-// stage_tma = 1) and bulk copies from the ghost-slab buffer (resolution
-// changes).
-__device__ __forceinline__ void mx_copy_masks(const StageArgs& a, const BlockDev& B, unsigned& tmask,
-                                              unsigned& amask) {
-  tmask = 0;
-  amask = 0;
+// What a block's six faces need (from its record): loaded ahead of the wait for
+// the tile.
+struct MxPlan {
+  int32_t ftype[6], fnb[6], rslot[6];
+};
+__device__ __forceinline__ MxPlan mx_plan(const StageArgs& a, int blk) {
+  MxPlan m;
+  const BlockDev& B = a.blocks[blk];
 #pragma unroll
   for (int f = 0; f < 6; f++) {
-    const int ft = B.ftype[f];
-    tmask |= (ft == FACE_SAME && a.stage_tma ? 1u : 0u) << f;
-    amask |= (ft == FACE_COARSER || ft == FACE_FINER ? 1u : 0u) << f;
+    m.ftype[f] = B.ftype[f];
+    m.fnb[f] = B.fnb[f];
+    m.rslot[f] = B.rslot[f];
   }
+  return m;
+}
+// Faces whose slabs no copy brings: outflow and inflow faces, and same-level
+// faces when stage_tma = 0.
+__device__ __forceinline__ unsigned mx_fill_mask(const StageArgs& a, const MxPlan& m) {
+  unsigned fill = 0;
+#pragma unroll
+  for (int f = 0; f < 6; f++)
+    fill |= (m.ftype[f] == FACE_OUTFLOW || m.ftype[f] == FACE_INFLOW || (m.ftype[f] == FACE_SAME && !a.stage_tma)
+                 ? 1u : 0u) << f;
+  return fill;
 }
 
-// Issue (one thread) the copies of block blk's tile on bar: the interior,
-// the copied face slabs.  Any generic-proxy access to sT that they overwrite
-// must be ordered before (the caller's barrier); this fences the proxies.
-__device__ __forceinline__ void mx_issue_copies(const StageArgs& a, const BlockDev& B, int blk, float* sT,
-                                                uint64_t* bar) {
-  unsigned tmask, amask;
-  mx_copy_masks(a, B, tmask, amask);
-  {
-    fence_proxy_async();
-    uint32_t bytes = NV * NCELL * 4;
+// Issue (one thread) the copies of block blk on bar: its record, the interior,
+// the copied face slabs (tensor copies at the same level, bulk copies from the
+// ghost-slab buffer at resolution changes).  Any generic-proxy access to sT that
+// they overwrite must be ordered before (the caller's barrier); this fences
+// the proxies.
+__device__ __forceinline__ void mx_issue_copies(const StageArgs& a, const MxPlan& m, unsigned fill, int blk, float* sT,
+                                                BlockDev* rec, uint64_t* bar) {
+  fence_proxy_async();
+  uint32_t bytes = NV * NCELL * 4 + sizeof(BlockDev);
 #pragma unroll
-    for (int f = 0; f < 6; f++)
-      if (((tmask | amask) >> f) & 1u) bytes += mx_slab_bytes(f >> 1);
-    mbar_expect_tx(bar, bytes);
-    tma_load_4d(sT, &a.tm[0], 0, 0, 0, blk * NV, bar);
+  for (int f = 0; f < 6; f++)
+    if (!((fill >> f) & 1u)) bytes += mx_slab_bytes(f >> 1);
+  mbar_expect_tx(bar, bytes);
+  tma_load_4d(sT, &a.tm[0], 0, 0, 0, blk * NV, bar);
 #pragma unroll
-    for (int f = 0; f < 6; f++) {
-      if ((tmask >> f) & 1u) {
-        const int nb = chki(B.fnb[f], 0, a.nblocks), d = f >> 1, side = f & 1;
-        // the neighbour's cells nearest the face: 4-7 / 0-3 along x, 6-7 / 0-1 along y and z
-        const int o = side ? 0 : (d == 0 ? 4 : 6);
-        tma_load_4d(sT + mx_slab_base(f), &a.tm[1 + d], d == 0 ? o : 0, d == 1 ? o : 0, d == 2 ? o : 0, nb * NV,
-                    bar);
-      } else if ((amask >> f) & 1u) {
-        const float* g = a.gbuf + chk(B.rslot[f], 0, a.nslots) * GSLOT;
-        bulk_g2s(sT + mx_slab_base(f), g, mx_slab_bytes(f >> 1), bar);
-      }
+  for (int f = 0; f < 6; f++) {
+    if ((fill >> f) & 1u) continue;
+    if (m.ftype[f] == FACE_SAME) {
+      const int nb = chki(m.fnb[f], 0, a.nblocks), d = f >> 1, side = f & 1;
+      // the neighbour's cells nearest the face: 4-7 / 0-3 along x, 6-7 / 0-1 along y and z
+      const int o = side ? 0 : (d == 0 ? 4 : 6);
+      tma_load_4d(sT + mx_slab_base(f), &a.tm[1 + d], d == 0 ? o : 0, d == 1 ? o : 0, d == 2 ? o : 0, nb * NV, bar);
+    } else {
+      bulk_g2s(sT + mx_slab_base(f), a.gbuf + chk(m.rslot[f], 0, a.nslots) * GSLOT, mx_slab_bytes(f >> 1), bar);
     }
   }
+  bulk_g2s(rec, &a.blocks[blk], sizeof(BlockDev), bar);
 }
 
-// The calling threads fill the face slabs of block blk that no copy brings:
-// outflow and inflow faces, and same-level faces when stage_tma = 0.
-__device__ __forceinline__ void mx_fill_slabs(const StageArgs& a, const BlockDev& B, int blk, float* sT, int tid,
+// The calling threads fill the face slabs `fill` of block B, its interior being
+// in the tile: an outflow ghost is the block's own boundary cell.
+__device__ __forceinline__ void mx_fill_slabs(const StageArgs& a, const BlockDev& B, unsigned fill, float* sT, int tid,
                                               int nthr) {
-  unsigned tmask, amask;
-  mx_copy_masks(a, B, tmask, amask);
-  const unsigned fill = 0x3fu & ~(tmask | amask);
   const int nfill = __popc(fill) * 128;
   for (int q = tid; q < nfill; q += nthr) {
     const int slot = q >> 7, loc = q & 127;
@@ -1468,9 +1465,22 @@ __device__ __forceinline__ void mx_fill_slabs(const StageArgs& a, const BlockDev
     for (int k = 0; k < slot; k++) m &= m - 1;
     const int s = __ffs(m) - 1, d = s >> 1, side = s & 1;
     const int layer = loc & 1, ta = (loc >> 1) & 7, tb = loc >> 4;
+    const int c = side ? NC + layer : layer - 2, ft = B.ftype[s];
     float w[8];
-    mx_ghost_value(a, a.grids[B.grid], B, blk, s, layer, ta, tb, w);
-    const int c = side ? NC + layer : layer - 2;
+    if (ft == FACE_INFLOW) {
+      const GridDev& G = a.grids[B.grid];
+#pragma unroll
+      for (int v = 0; v < NV; v++) w[v] = G.Winflow32[v];
+    } else {
+      const int cn = ft == FACE_SAME ? (side ? c - NC : c + NC) : (side ? NC - 1 : 0);
+      const int i = d == 0 ? cn : ta, j = d == 1 ? cn : (d == 0 ? ta : tb), k = d == 2 ? cn : tb;
+      const int cell = chki((k * NC + j) * NC + i, 0, NCELL);
+      const float* p = ft == FACE_SAME
+                           ? a.Win + static_cast<int64_t>(chki(B.fnb[s], 0, a.nblocks)) * (NV * NCELL) + cell
+                           : sT + mx_int(cell);
+#pragma unroll
+      for (int v = 0; v < NV; v++) w[v] = p[v * NCELL];
+    }
     float* o = sT + mx_slab_base(s) + chki(mx_slab_elem(d, side, c, ta, tb), 0, mx_slab_vstride(d));
     const int vs = mx_slab_vstride(d);
 #pragma unroll
@@ -1478,20 +1488,14 @@ __device__ __forceinline__ void mx_fill_slabs(const StageArgs& a, const BlockDev
   }
 }
 
-// Stage block blk into the tile sT: copies issued by thread 0 on bar, the
-// remaining slabs filled by the calling threads.  Returns after the fill;
-// the caller waits on bar and synchronises.
-__device__ __forceinline__ void mx_stage_tile(const StageArgs& a, const BlockDev& B, int blk, float* sT,
-                                              uint64_t* bar, int tid, int nthr) {
-  if (tid == 0) mx_issue_copies(a, B, blk, sT, bar);
-  mx_fill_slabs(a, B, blk, sT, tid, nthr);
-}
-
 // The faces of one direction D on this thread's grid line for the staged
-// tile: lane half 0 walks up from cell -2 (faces 0-4), half 1 walks down from
-// cell 9 (faces 8-5; its fifth step is face 4, computed by half 0, and not
-// stored), so that at every step both halves read the same kind of cell (two
-// ghost cells, then interior cells) with the same variable stride.  Walking
+// tile: half 0 walks up from cell -2 (faces 0-4), half 1 walks down from cell 9
+// (faces 8-5), so that at every step both halves read the same kind of cell
+// (two ghost cells, then interior cells) with the same variable stride.  y, z:
+// the halves of a line belong to different warps (a warp takes 5 or 4 steps as
+// a whole, and its 32 lanes read 32 different banks).  x: a warp's even lanes
+// take half 0 and its odd lanes half 1 (its 32 lines at one cell would meet on 8
+// banks, two cells halve that); its fifth step of half 1 is thrown away.  Walking
 // down, a face's two sides come as (right, left): the dissipation's sign
 // flips with the lane's direction.  Writes twice the fluxes (un-rotated
 // components) and the sum of the two sides' normal B1 into sF[D][9][576].
@@ -1516,11 +1520,9 @@ __device__ __forceinline__ void faces_mx(const int D, const StageArgs& a, const 
   const int fta = fline & 7, ftb = fline >> 3;
   const bool h1 = fhalf != 0;
   // interior index of cell c along the line
-  auto cint = [&](int c) -> int {
-    if (D == 0) return mx_int(c, fta, ftb);
-    if (D == 1) return mx_int(fta, c, ftb);
-    return mx_int(fta, ftb, c);
-  };
+  const int clin = D == 0 ? 64 * ftb + 8 * fta : (D == 1 ? 64 * ftb + fta : 8 * ftb + fta);
+  const int cstr = D == 0 ? 1 : (D == 1 ? NC : NC * NC);
+  auto cint = [&](int c) -> int { return mx_int(clin + c * cstr); };
   // window step j: half 0 cell j - 2, half 1 cell 9 - j
   auto cell_of = [&](int j) -> int { return h1 ? 9 - j : j - 2; };
   const int gbase = (h1 ? (D == 0 ? MX_GX1 : D == 1 ? MX_GY1 : MX_GZ1) : (D == 0 ? MX_GX0 : D == 1 ? MX_GY0 : MX_GZ0));
@@ -1552,6 +1554,7 @@ __device__ __forceinline__ void faces_mx(const int D, const StageArgs& a, const 
   const float dsgn = h1 ? -1.f : 1.f;
 #pragma unroll
   for (int k = 0; k < 5; k++) {
+    if (k == 4 && D != 0 && h1) break;  // half 1's faces are done (warp-uniform)
     float Wp[8];
     load_i(k + 3, Wp);
     float2 W2[8];
@@ -1609,16 +1612,17 @@ __device__ __forceinline__ void faces_mx(const int D, const StageArgs& a, const 
 // Returns this thread's largest CFL bound (last stage), 0 otherwise.
 // The pair's primitives Wc (the stage input) come from the tile, read by the
 // caller before the next block's copies overwrite it (first stage only: the
-// last stage reads them, for the Powell term, from memory).
+// last stage reads them, for the Powell term, from memory); the grid's dt is
+// loaded by the caller ahead of the wait for the faces.
 __device__ __forceinline__ void cells_mx_pair_w(const float* sT, int tid, float2 Wc[8]) {
   if (tid >= NCELL / 2) return;
-  const int cs = tid ^ (((tid >> 5) & 1) << 2);  // the interior's swizzle (the pair shares it)
+  const int cs = mx_int(tid);  // the interior's swizzle (the pair shares it)
 #pragma unroll
   for (int v = 0; v < NV; v++) Wc[v] = make_float2(sT[v * NCELL + cs], sT[v * NCELL + cs + NCELL / 2]);
 }
 __device__ __forceinline__ float cells_mx_pair(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk,
-                                               const float2 Wc[8], const float* sF, int tid, float fx, float fy,
-                                               float fz, float idx0, float idx1, float idx2, float gamma) {
+                                               const float2 Wc[8], double dtg, const float* sF, int tid, float fx,
+                                               float fy, float fz, float idx0, float idx1, float idx2, float gamma) {
   if (tid >= NCELL / 2) return 0.f;
   const PhysDev& ph = a.ph;
   const int c = tid, ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6;  // ck 0..3; the pair's second cell: ck + 4
@@ -1672,7 +1676,7 @@ __device__ __forceinline__ float cells_mx_pair(const StageArgs& a, const GridDev
     }
     R[7] = p_fma(nd, ub1, R[7]);
   }
-  const double cdt = a.beta * a.dt[B.grid];
+  const double cdt = a.beta * dtg;
   if (light) {
     // first midpoint stage: W* = W^n + the increment, in FP32
     const float c32 = d2f_int(cdt);
@@ -1786,6 +1790,354 @@ __device__ __forceinline__ float cells_mx_pair(const StageArgs& a, const GridDev
     m = fmaxf(sacc.x, sacc.y);
   }
   return m;
+}
+
+// Mixed plain kernel, every other case (SSP-RK2, local time steps, blocks with
+// body cells, a background field, the residual view): one cell per thread and
+// turn over the nthr calling threads.  FAST (compile time): kind 0, no local
+// time steps, no body cell in the block (GB300 runs FP64 at 1/64 of the FP32
+// rate, so even FP64 instructions issued predicated off cost).  Returns this
+// thread's largest CFL bound (last stage).
+template <bool HAS_B0, bool FAST>
+__device__ __forceinline__ float cells_mx_general(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk,
+                                                  const float* sT, const float* sF, int tid, int nthr, double dtg) {
+  const PhysDev& ph = a.ph;
+  const int kind = FAST ? 0 : a.kind;
+  double* const dtc = FAST ? nullptr : a.dtc;
+  const bool blk_body = FAST ? false : B.body != 0;
+  const float idx0 = B.idxf[0], idx1 = B.idxf[1], idx2 = B.idxf[2];
+  const float dxr0 = B.dxf[0], dxr1 = B.dxf[1], dxr2 = B.dxf[2];
+  const float lor0 = G.lof[0], lor1 = G.lof[1], lor2 = G.lof[2];
+  const int gb0 = B.bi * NC, gb1 = B.bj * NC, gb2 = B.bk * NC, lev = B.level;
+  const float gamma = ph.gammaf;
+  // the face values are doubled
+  const float fidx0 = 0.5f * idx0, fidx1 = 0.5f * idx1, fidx2 = 0.5f * idx2;
+  float smax_loc = 0.f;
+  const double cdt_blk = a.beta * dtg;
+  // first stage of the midpoint scheme: U* only feeds the second stage's FP32
+  // primitives, so W* = W^n + the increment, in FP32 (the FP64 state is read
+  // and accumulated in the last stage only)
+  const bool light = kind == 0 && !a.last && !a.write_u_all;
+  const float c32_blk = d2f_int(cdt_blk);
+  for (int c = tid; c < NCELL; c += nthr) {
+    // local time stepping: this cell's own dt
+    const double cdt = dtc ? a.beta * dtc[static_cast<int64_t>(blk) * NCELL + c] : cdt_blk;
+    const float c32 = dtc ? d2f_int(cdt) : c32_blk;
+    const int ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6;
+    // face indices (line * 9 + position) of the low faces in x, y, z
+    const int tx = chki((ck * NC + cj) * 9 + ci, 0, NFACE - 1);
+    const int ty = chki((ck * NC + ci) * 9 + cj, 0, NFACE - 1);
+    const int tz = chki((cj * NC + ci) * 9 + ck, 0, NFACE - 1);
+    const float* Fx = sF;
+    const float* Fy = sF + 9 * NFACE;
+    const float* Fz = sF + 2 * 9 * NFACE;
+    float res[8];
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const int vx = frot(v, 0) * NFACE, vy = frot(v, 1) * NFACE, vz = frot(v, 2) * NFACE;  // face-frame slots
+      float r = -((Fx[vx + tx + 1] - Fx[vx + tx]) * fidx0);
+      r = r - (Fy[vy + ty + 1] - Fy[vy + ty]) * fidx1;
+      r = r - (Fz[vz + tz + 1] - Fz[vz + tz]) * fidx2;
+      res[v] = r;
+    }
+    const float divb = ((Fx[8 * NFACE + tx + 1] - Fx[8 * NFACE + tx]) * fidx0 +
+                        (Fy[8 * NFACE + ty + 1] - Fy[8 * NFACE + ty]) * fidx1) +
+                       (Fz[8 * NFACE + tz + 1] - Fz[8 * NFACE + tz]) * fidx2;
+    bool in_body = false;
+    if (blk_body) {  // FP64, the same centre formula as the host and the oracle
+      double x = G.lo[0] + ((static_cast<double>(gb0) + ci) + 0.5) * G.dx[lev][0];
+      double y = G.lo[1] + ((static_cast<double>(gb1) + cj) + 0.5) * G.dx[lev][1];
+      double z = G.lo[2] + ((static_cast<double>(gb2) + ck) + 0.5) * G.dx[lev][2];
+      in_body = (x * x + y * y + z * z) < G.body_r * G.body_r;
+    }
+    float Wc[8];
+#pragma unroll
+    for (int v = 0; v < NV; v++) Wc[v] = sT[v * NCELL + mx_int(c)];
+    float B0c[3] = {0.f, 0.f, 0.f};
+    float S[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if constexpr (HAS_B0) b0_face<float>(ph, -1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, B0c);
+    if (ph.powell) {
+      float ub1 = Wc[1] * Wc[4] + Wc[2] * Wc[5] + Wc[3] * Wc[6];
+#pragma unroll
+      for (int e = 0; e < 3; e++) {
+        S[1 + e] = -divb * (B0c[e] + Wc[4 + e]);
+        S[4 + e] = -divb * Wc[1 + e];
+      }
+      S[7] = -divb * ub1;
+    }
+    if constexpr (HAS_B0) {
+      // split-field correction from the face-centre B0 of the six faces:
+      // S_m += -B1 (div B0)_h + B1 x (curl B0)_h
+      float xm[3], xp[3], ym[3], yp[3], zm[3], zp[3];
+      b0_face<float>(ph, 0, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xm);
+      b0_face<float>(ph, 0, ci + 1, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xp);
+      b0_face<float>(ph, 1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, ym);
+      b0_face<float>(ph, 1, ci, cj + 1, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, yp);
+      b0_face<float>(ph, 2, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zm);
+      b0_face<float>(ph, 2, ci, cj, ck + 1, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zp);
+      float divb0 = ((xp[0] - xm[0]) * idx0 + (yp[1] - ym[1]) * idx1) + (zp[2] - zm[2]) * idx2;
+      float cu0 = (yp[2] - ym[2]) * idx1 - (zp[1] - zm[1]) * idx2;
+      float cu1 = (zp[0] - zm[0]) * idx2 - (xp[2] - xm[2]) * idx0;
+      float cu2 = (xp[1] - xm[1]) * idx0 - (yp[0] - ym[0]) * idx1;
+      float b1x = Wc[4], b1y = Wc[5], b1z = Wc[6];
+      S[1] = (S[1] - b1x * divb0) + (b1y * cu2 - b1z * cu1);
+      S[2] = (S[2] - b1y * divb0) + (b1z * cu0 - b1x * cu2);
+      S[3] = (S[3] - b1z * divb0) + (b1x * cu1 - b1y * cu0);
+    }
+    const int64_t base = static_cast<int64_t>(blk) * (NV * NCELL) + c;
+    if (light) {
+      float dU[8], Wl[8];
+#pragma unroll
+      for (int v = 0; v < NV; v++) dU[v] = c32 * (res[v] + S[v]);
+      prim_increment(Wc, dU, ph.gm1f, Wl);
+      if (in_body) prim_mixed(G.Ubody, ph.gm1f, Wl);
+      bool badl = !(Wl[0] > 0.f) || !(Wl[7] > 0.f);
+#pragma unroll
+      for (int v = 0; v < NV; v++) badl |= !finite_f(Wl[v]);
+      if (badl && !in_body) {
+        atomicOr(&a.err[0], ERR_NONPHYSICAL);
+        atomicMin(&a.err[1], blk);
+      }
+#pragma unroll
+      for (int v = 0; v < NV; v++) a.Wout[base + v * NCELL] = Wl[v];
+      continue;
+    }
+    double Uo[8];
+    bool bad = false;
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const double rd = f2d_int(res[v] + S[v]);
+      double ub = a.Ubase[base + v * NCELL];
+      double o;
+      if (kind == 0) o = fma(cdt, rd, ub);
+      else o = 0.5 * ub + 0.5 * fma(cdt, rd, a.Uin[base + v * NCELL]);
+      if (kind == 2) o = rd;  // residual only (debug view)
+      Uo[v] = o;
+    }
+    if (in_body) {  // a branch, not a select: no loads of the body state elsewhere
+#pragma unroll
+      for (int v = 0; v < NV; v++) Uo[v] = kind == 2 ? 0.0 : G.Ubody[v];
+    }
+#pragma unroll
+    for (int v = 0; v < NV; v++) bad |= !finite_d(Uo[v]);
+    if (kind != 2) bad |= !positive_d(Uo[0]);
+    float Wn[8];
+    if (kind != 2) {
+      double p64;
+      prim_mixed(Uo, ph.gm1f, Wn, &p64);
+      bad |= !positive_d(p64);
+    }
+    if (bad && !in_body && kind != 2) {
+      atomicOr(&a.err[0], ERR_NONPHYSICAL);
+      atomicMin(&a.err[1], blk);
+    }
+    if (a.last || a.write_u_all || kind == 2) {
+#pragma unroll
+      for (int v = 0; v < NV; v++) a.Uout[base + v * NCELL] = Uo[v];
+    }
+    if (kind != 2) {
+#pragma unroll
+      for (int v = 0; v < NV; v++) a.Wout[base + v * NCELL] = Wn[v];
+    }
+    // CFL bound of the new state: sum_d (|u_d| + c_f,d) / dx_d (cells that
+    // refluxing corrects afterwards are bounded by the correction kernel)
+    const bool refl = a.freg && ((ci == 0 && B.ftype[0] == FACE_FINER) || (ci == NC - 1 && B.ftype[1] == FACE_FINER) ||
+                                 (cj == 0 && B.ftype[2] == FACE_FINER) || (cj == NC - 1 && B.ftype[3] == FACE_FINER) ||
+                                 (ck == 0 && B.ftype[4] == FACE_FINER) || (ck == NC - 1 && B.ftype[5] == FACE_FINER));
+    if (a.last && !in_body && kind != 2 && !refl) {
+      float Bt[3] = {B0c[0] + Wn[4], B0c[1] + Wn[5], B0c[2] + Wn[6]};
+      float sacc = 0.f;
+#pragma unroll
+      for (int e = 0; e < 3; e++) {
+        const float cf = fast_speed_n(gamma, Wn[0], Wn[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
+        sacc = sacc + (fabsf(Wn[1 + e]) + cf) * (e == 0 ? idx0 : (e == 1 ? idx1 : idx2));
+      }
+      smax_loc = sacc > smax_loc ? sacc : smax_loc;
+      if (dtc) dtc[static_cast<int64_t>(blk) * NCELL + c] = a.cfl / f2d_int(sacc);
+    } else if (a.last && dtc && kind != 2 && in_body) {
+      dtc[static_cast<int64_t>(blk) * NCELL + c] = 0.0;  // body cell
+    }
+  }
+  return smax_loc;
+}
+
+// The stage kernel of the plain mixed form, one CTA of 24 warps per SM walking
+// over its blocks.  What bounds it is latency: a block's faces and cells are long
+// dependent chains, and with every warp doing faces, then cells behind CTA-wide
+// barriers (two CTAs per SM), the schedulers issued on 47-55 % of the cycles,
+// the cells taking as long as the faces on two thirds of the warps.  Here the
+// warps are specialised, so that the phases of neighbouring blocks overlap and
+// the copies run a block ahead: 61 % of the cycles; 8 grids (3.1 M cells), stage
+// 1 169 -> 147 us, stage 2 (FP64 accumulation) 216 -> 178 us.
+//  * 12 face warps: faces_mx of one block after the other;
+//  * 12 cell warps: the cells of the blocks before, 1/8 of a block at a time in
+//    turn (a block's eight parts go to eight of the warps, the next block's to
+//    the other four and on): with eight warps a block's cells took twice as long
+//    as its faces in the last stage (long chains of shared-memory loads, FP64
+//    operations at 64 cycles per warp and global loads).  The warp with a block's first part also issues the copies of the
+//    next block's record and tile.
+// Tile q & 1 and face values q & 1 belong to the CTA's q-th block; they are
+// handed over through mbarriers: full (copies landed; faces done by the 12
+// warps) and empty (tile read by the 12 face warps and the 8 parts; face values
+// read by the 8 parts).  Shared memory (2 x (48 + 61) KB) bounds the depth.
+// Every wait is bounded: a warp whose wait ran out flags it, skips its work and
+// further waits from then on, but keeps arriving, so that every warp ends.
+constexpr int MX_PARTS = 8;
+struct MxBars {
+  uint64_t tile_full[2], tile_empty[2], face_full[2], face_empty[2], slabs[2];
+};
+template <int LIM, bool HAS_B0, int FLX>
+__global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constant__ StageArgs a) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  __shared__ MxBars bar;
+  __shared__ BlockDev rec[4];   // the records of the CTA's blocks, four deep (a tile's record outlives the tile)
+  __shared__ uint32_t fillm[4];  // their faces filled by threads
+  float* const sT = reinterpret_cast<float*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+  float* const sF = sT + 2 * MX_TILE;
+  constexpr int FACES = 3 * 9 * NFACE;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const PhysDev& ph = a.ph;
+  if (tid == 0) {
+#pragma unroll
+    for (int b = 0; b < 2; b++) {
+      mbar_init(&bar.tile_full[b], 1);
+      mbar_init(&bar.tile_empty[b], MX_FACE_WARPS + MX_PARTS);
+      mbar_init(&bar.face_full[b], MX_FACE_WARPS);
+      mbar_init(&bar.face_empty[b], MX_PARTS);
+      mbar_init(&bar.slabs[b], MX_FACE_WARPS);
+    }
+  }
+  __syncthreads();
+  const int nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
+  bool failed = false;
+  auto wait = [&](uint64_t* b, uint32_t parity) {
+    if (!failed) failed = !mbar_wait_inline(b, parity, a.err);
+  };
+  // two barriers, the first polls in flight together
+  auto wait2 = [&](uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, bool second) {
+    const bool r0 = mbar_try_wait(b0, p0), r1 = !second || mbar_try_wait(b1, p1);
+    if (!failed && !r0) failed = !mbar_wait_inline(b0, p0, a.err);
+    if (!failed && !r1) failed = !mbar_wait_inline(b1, p1, a.err);
+  };
+  // the CTA's n blocks: items of bpi consecutive blocks, every gridDim.x-th one
+  const int bpi = a.blocks_per_item;
+  const int items = static_cast<int>(blockIdx.x) < nitems ? (nitems - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1 : 0;
+  const bool has_last = items > 0 && (static_cast<int>(blockIdx.x) + (items - 1) * static_cast<int>(gridDim.x)) == nitems - 1;
+  const int n = items * bpi - (has_last ? nitems * bpi - a.nblocks : 0);
+  auto block_of = [&](int q) {
+    const int it = q / bpi;
+    return (static_cast<int>(blockIdx.x) + it * static_cast<int>(gridDim.x)) * bpi + (q - it * bpi);
+  };
+  // one thread: the copies of the CTA's q-th block, once its tile is free
+  const bool reads_ubase = !(a.kind == 0 && !a.last && !a.write_u_all);
+  auto issue = [&](int q) {
+    const int b = q & 1, blk = block_of(q);
+    const MxPlan plan = mx_plan(a, blk);
+    const unsigned fill = mx_fill_mask(a, plan);
+    if (q >= 2) wait(&bar.tile_empty[b], ((q >> 1) - 1) & 1);
+    if (failed) return;  // nothing more is copied
+    fillm[q & 3] = fill;
+    mx_issue_copies(a, plan, fill, blk, sT + b * MX_TILE, &rec[q & 3], &bar.tile_full[b]);
+    // the FP64 states the cell warps read, on their way to L2 meanwhile
+    const int64_t boff = static_cast<int64_t>(blk) * (NV * NCELL);
+    if (reads_ubase) prefetch_l2(a.Ubase + boff, NV * NCELL * sizeof(double));
+    if (a.kind == 1) prefetch_l2(a.Uin + boff, NV * NCELL * sizeof(double));
+  };
+
+  if (warp < MX_FACE_WARPS) {
+    // four warps per direction (warp-uniform).  y and z: 32 lines of one half
+    // per warp; x: a line's two halves in neighbouring lanes
+    const int fd = warp >> 2;
+    const int fline = fd != 0 ? 32 * (warp & 1) + lane : 16 * (warp & 3) + (lane >> 1);
+    const int fhalf = fd != 0 ? (warp >> 1) & 1 : lane & 1;
+    uint32_t nslabs = 0;  // blocks with slabs filled by threads so far, per buffer (bits 0, 1: parity)
+    for (int q = 0; q < n; q++) {
+      const int b = q & 1;
+      float* const tile = sT + b * MX_TILE;
+      wait2(&bar.tile_full[b], (q >> 1) & 1, &bar.face_empty[b], ((q >> 1) - 1) & 1, q >= 2);
+      const BlockDev& B = rec[q & 3];
+      const uint32_t fill = failed ? 0u : fillm[q & 3];
+      if (fill) {
+        mx_fill_slabs(a, B, fill, tile, tid, 32 * MX_FACE_WARPS);
+        // the slabs no copy brings: complete when all face warps have filled theirs
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar.slabs[b]);
+        wait(&bar.slabs[b], (nslabs >> b) & 1);
+        nslabs ^= 1u << b;
+      }
+      if (!failed) {
+        const GridDev& G = a.grids[B.grid];
+        faces_mx<LIM, HAS_B0, FLX>(fd, a, B, tile, sF + b * FACES, fline, fhalf, ph.gammaf, ph.inv_gm1f, B.bi * NC,
+                                   B.bj * NC, B.bk * NC, HAS_B0 ? G.lof[0] : 0.f, HAS_B0 ? G.lof[1] : 0.f,
+                                   HAS_B0 ? G.lof[2] : 0.f, B.dxf[0], B.dxf[1], B.dxf[2]);
+      }
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&bar.face_full[b]);
+        mbar_arrive(&bar.tile_empty[b]);
+      }
+    }
+    return;
+  }
+
+  const int cw = warp - MX_FACE_WARPS;
+  if (cw == 0 && lane == 0 && n > 0) issue(0);
+  for (int part = cw; part < MX_PARTS * n; part += MX_CELL_WARPS) {
+    const int q = part / MX_PARTS, b = q & 1, blk = block_of(q);
+    const int ct = 32 * (part % MX_PARTS) + lane;  // 0..255: cells ct and ct + 256
+    if (part % MX_PARTS == 0 && q + 1 < n) {
+      if (lane == 0) issue(q + 1);
+      failed = __shfl_sync(0xffffffffu, failed, 0);
+    }
+    const float* const tile = sT + b * MX_TILE;
+    const float* const F = sF + b * FACES;
+    wait(&bar.tile_full[b], (q >> 1) & 1);
+    const BlockDev& B = rec[q & 3];
+    const bool fast = !failed && !HAS_B0 && a.kind == 0 && !a.dtc && !B.body;
+    const bool light = !a.last && !a.write_u_all;
+    double dtg = 0.0;
+    float2 Wc[8];
+    if (!failed) dtg = a.kind == 2 ? 0.0 : ld_early(a.dt + B.grid);
+    if (fast) {
+      if (light) cells_mx_pair_w(tile, ct, Wc);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar.tile_empty[b]);
+    }
+    wait(&bar.face_full[b], (q >> 1) & 1);
+    float m = 0.f;
+    if (!failed) {
+      const GridDev& G = a.grids[B.grid];
+      if constexpr (HAS_B0) {
+        m = a.kind == 0 && !a.dtc && !B.body
+                ? cells_mx_general<HAS_B0, true>(a, G, B, blk, tile, F, ct, 32 * MX_PARTS, dtg)
+                : cells_mx_general<HAS_B0, false>(a, G, B, blk, tile, F, ct, 32 * MX_PARTS, dtg);
+      } else {
+        m = fast ? cells_mx_pair(a, G, B, blk, Wc, dtg, F, ct, 0.5f * B.idxf[0], 0.5f * B.idxf[1],
+                                 0.5f * B.idxf[2], B.idxf[0], B.idxf[1], B.idxf[2], ph.gammaf)
+                 : cells_mx_general<HAS_B0, false>(a, G, B, blk, tile, F, ct, 32 * MX_PARTS, dtg);
+      }
+    }
+    if (a.last && a.kind != 2) {
+      // this warp's largest bound: the bits of non-negative floats order like
+      // the floats
+      const uint32_t mw = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+      if (lane == 0 && mw != 0u)
+        atomicMax(&a.smax_next[B.grid],
+                  static_cast<unsigned long long>(__double_as_longlong(f2d_int(__uint_as_float(mw)))));
+    }
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(&bar.face_empty[b]);
+      if (!fast) mbar_arrive(&bar.tile_empty[b]);
+    }
+  }
+  // after a failure no copy stays in flight into this CTA's shared memory
+  // (otherwise the warps have waited for all of them)
+  if (failed)
+    for (int b = 0; b < 2; b++) {
+      mbar_wait_inline(&bar.tile_full[b], 0, a.err);
+      mbar_wait_inline(&bar.tile_full[b], 1, a.err);
+    }
 }
 
 constexpr int TC_TILE_F = 128;  // rows per tensor-core tile (MMA M = tensor-memory lanes)
@@ -1952,30 +2304,22 @@ __device__ __forceinline__ bool lrn_network(LrnSmem& s, const uint4 xrow[6], flo
   return true;
 }
 
-// The fused stage (StageCfg::THREADS threads).  Per block: (1) interior by TMA, face-slab
-// ghosts by threads; (2) FP64 form: primitives in place; (3) faces of all
+// The fused stage of the FP64 form and of the learned correction in the mixed form
+// (the plain mixed one: k_stage_mx below), one CTA of 384 threads per SM.  Per
+// block: (1) interior by TMA, face-slab ghosts by threads; (2) FP64 form: primitives in place; (3) faces of all
 // three directions at once on the first FACE_THREADS threads, two per grid
 // line (faces 0-4 and 5-8), each sliding a window along its line so that
 // every cell is loaded and every limited slope computed once; (4) per cell:
 // flux differences x, y, z, the sources, the update and (last stage) the CFL
 // bound.
 template <bool MIXED, int LIM, bool HAS_B0, bool LRN, int FLX>
-__global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 : 1)
-    k_stage(const __grid_constant__ StageArgs a) {
+__global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constant__ StageArgs a) {
+  static_assert(!MIXED || LRN, "the plain mixed stage is k_stage_mx");
   using R = typename StageCfg<MIXED>::R;
-  constexpr int STAGE_THREADS = StageCfg<MIXED>::THREADS;
   constexpr int NFC = StageCfg<MIXED>::NFC;
-  // mixed form without the learned correction: the staged tile (tensor copies)
-  constexpr bool MX = MIXED && !LRN;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  R* sT;                                         // tile: [8][1280] (generic) or the staged layout (MX)
-  if constexpr (MX) {
-    const uint32_t pad = (1024u - (smem_u32(smem_raw) & 1023u)) & 1023u;
-    sT = reinterpret_cast<R*>(smem_raw + pad);
-  } else {
-    sT = reinterpret_cast<R*>(smem_raw);
-  }
-  R* sF = sT + (MX ? MX_TILE : NV * NTILE);      // [3][9][576] face values
+  R* sT = reinterpret_cast<R*>(smem_raw);        // tile [8][1280]
+  R* sF = sT + NV * NTILE;                       // [3][9][576] face values
   // mixed learned kernel: the network runs fused, on the tensor cores
   constexpr bool LX = MIXED && LRN;
   LrnSmem* ls = nullptr;
@@ -2031,13 +2375,6 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
   uint32_t parity = 0;
 
   const int nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
-  if constexpr (MX) {
-    // the staged tile's copies run one block ahead: those of each block are
-    // issued while the block before it is in its cell phase (which reads the
-    // face values and global memory only); the first block's here
-    const int b0 = blockIdx.x * a.blocks_per_item;
-    if (tid == 0 && b0 < a.nblocks) mx_issue_copies(a, a.blocks[b0], b0, reinterpret_cast<float*>(sT), &bar);
-  }
   for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
     const int b_end = min(a.nblocks, (item + 1) * a.blocks_per_item);
     for (int blk = item * a.blocks_per_item; blk < b_end; blk++) {
@@ -2045,10 +2382,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
       const GridDev& G = a.grids[B.grid];
       GhostCtx cx{&G, a.blocks, a.levmap, a.Uin, a.err};
 
-      // 1. interior by TMA bulk copies (one per variable), ghosts by threads;
-      //    the mixed plain kernel: the staged tile (tensor copies)
-      if constexpr (MX) mx_fill_slabs(a, B, blk, reinterpret_cast<float*>(sT), tid, STAGE_THREADS);
-      if (tid == 0 && !MX) {
+      // 1. interior by TMA bulk copies (one per variable), ghosts by threads
+      if (tid == 0) {
         fence_proxy_async();
         // mixed form: the ghost slabs of faces at resolution changes come
         // precomputed, by bulk copies on the same barrier
@@ -2088,12 +2423,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
         if (reads_ubase) prefetch_l2(a.Ubase + boff, NV * NCELL * sizeof(double));
         if (MIXED && a.kind == 1) prefetch_l2(a.Uin + boff, NV * NCELL * sizeof(double));
       }
-      if constexpr (MX) {
-      } else if constexpr (MIXED) {
-        fill_ghosts_block_mixed(a, cx, B, blk, sT, tid, STAGE_THREADS, false);
-      } else {
-        fill_ghosts_block<false, double>(a, cx, B, blk, sT, sF, tid, STAGE_THREADS);
-      }
+      if constexpr (MIXED) fill_ghosts_block_mixed(a, cx, B, blk, sT, tid, STAGE_THREADS, false);
+      else fill_ghosts_block<false, double>(a, cx, B, blk, sT, sF, tid, STAGE_THREADS);
       if (!mbar_wait_bounded(&bar, parity, a.err)) mbar_wait_bounded(&bar, parity, a.err);
       parity ^= 1u;
       __syncthreads();
@@ -2116,8 +2447,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
       const int lev = B.level;
       R idx0, idx1, idx2, dxr0, dxr1, dxr2, lor0, lor1, lor2;
       if constexpr (MIXED) {
-        idx0 = G.idxf[lev][0]; idx1 = G.idxf[lev][1]; idx2 = G.idxf[lev][2];
-        dxr0 = G.dxf[lev][0]; dxr1 = G.dxf[lev][1]; dxr2 = G.dxf[lev][2];
+        idx0 = B.idxf[0]; idx1 = B.idxf[1]; idx2 = B.idxf[2];
+        dxr0 = B.dxf[0]; dxr1 = B.dxf[1]; dxr2 = B.dxf[2];
         lor0 = G.lof[0]; lor1 = G.lof[1]; lor2 = G.lof[2];
       } else {
         idx0 = G.idx[lev][0]; idx1 = G.idx[lev][1]; idx2 = G.idx[lev][2];
@@ -2347,7 +2678,7 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
         // mixed form, first stage of the midpoint scheme: U* only feeds the
         // second stage's FP32 primitives, so W* = W^n + the increment, in FP32
         // (the FP64 state is read and accumulated in the last stage only)
-        const bool light = MIXED && kind == 0 && !a.last && !a.write_u_all;
+        [[maybe_unused]] const bool light = MIXED && kind == 0 && !a.last && !a.write_u_all;
         const float c32_blk = d2f_int(cdt_blk);
         for (int c = tid; c < NCELL; c += STAGE_THREADS) {
           // local time stepping: this cell's own dt
@@ -2364,15 +2695,13 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
           R res[8];
 #pragma unroll
           for (int v = 0; v < NV; v++) {
-            // the mixed plain kernel's face values are in the face frame (frot)
-            const int vx = MX ? frot(v, 0) : v, vy = MX ? frot(v, 1) : v, vz = MX ? frot(v, 2) : v;
-            R r = -((Fx[vx * NFACE + tx + 1] - Fx[vx * NFACE + tx]) * fidx0);
-            r = r - (Fy[vy * NFACE + ty + 1] - Fy[vy * NFACE + ty]) * fidx1;
-            r = r - (Fz[vz * NFACE + tz + 1] - Fz[vz * NFACE + tz]) * fidx2;
+            R r = -((Fx[v * NFACE + tx + 1] - Fx[v * NFACE + tx]) * fidx0);
+            r = r - (Fy[v * NFACE + ty + 1] - Fy[v * NFACE + ty]) * fidx1;
+            r = r - (Fz[v * NFACE + tz + 1] - Fz[v * NFACE + tz]) * fidx2;
             res[v] = r;
           }
           R divb = R(0);
-          if (MX || ph.powell)
+          if (MIXED || ph.powell)
             divb = ((Fx[8 * NFACE + tx + 1] - Fx[8 * NFACE + tx]) * fidx0 +
                     (Fy[8 * NFACE + ty + 1] - Fy[8 * NFACE + ty]) * fidx1) +
                    (Fz[8 * NFACE + tz + 1] - Fz[8 * NFACE + tz]) * fidx2;
@@ -2384,14 +2713,8 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
             in_body = (x * x + y * y + z * z) < G.body_r * G.body_r;
           }
           R Wc[8];
-          if constexpr (MX) {
-            const int cs = c ^ (((c >> 5) & 1) << 2);  // the interior's swizzle (j >= 4: halves exchanged)
 #pragma unroll
-            for (int v = 0; v < NV; v++) Wc[v] = sT[v * NCELL + cs];
-          } else {
-#pragma unroll
-            for (int v = 0; v < NV; v++) Wc[v] = sT[v * NTILE + c];
-          }
+          for (int v = 0; v < NV; v++) Wc[v] = sT[v * NTILE + c];
           R B0c[3] = {R(0), R(0), R(0)};
           R S[8] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
           if constexpr (HAS_B0) b0_face<R>(ph, -1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, B0c);
@@ -2551,13 +2874,7 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
         return any_bad;
       };
 
-      if constexpr (MX) {
-        // one direction per warp group (fd is warp-uniform)
-        if (tid < FACE_THREADS) {
-          faces_mx<LIM, HAS_B0, FLX>(fd, a, B, sT, sF, fline, fhalf, gamma, inv_gm1, gb0, gb1, gb2, lor0, lor1, lor2,
-                                     dxr0, dxr1, dxr2);
-        }
-      } else if constexpr (!LRN) {
+      if constexpr (!LRN) {
         // half h of the lines 32 (w & 1) .. of direction fd per warp w of its
         // four; the halves' order alternates over the directions, so that the
         // SM's four schedulers get 13 or 14 of the 54 warp steps each
@@ -2570,52 +2887,17 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
       } else {
         if (tid < FACE_THREADS) faces(true);
       }
-      // a tensor-core wait ran out in some warp group: the error is flagged, stop
-      if (__syncthreads_or(mfail)) {
-        mfail = true;
-        break;
-      }
-      // the staged tile's next block (its copies go out once this block's
-      // cell phase has read what it needs from the tile)
-      const int nblk = blk + 1 < b_end ? blk + 1 : (item + static_cast<int>(gridDim.x)) * a.blocks_per_item;
-      // issuer: a thread of a warp with no cell work in the packed cell phase
-      // (threads 256-383), so that its wait for the next block's table entry
-      // delays no cell's update
-      auto issue_next = [&](int issuer) {
-        if constexpr (MX) {
-          if (tid == issuer && nblk < a.nblocks)
-            mx_issue_copies(a, a.blocks[nblk], nblk, reinterpret_cast<float*>(sT), &bar);
+      if constexpr (LX) {
+        // a tensor-core wait ran out in some warp group: the error is flagged, stop
+        if (__syncthreads_or(mfail)) {
+          mfail = true;
+          break;
         }
-      };
+      } else {
+        __syncthreads();
+      }
       if (a.kind >= 3) continue;  // features / dumps only
       const bool fast = a.kind == 0 && !a.dtc && !B.body;
-      if constexpr (MX && !HAS_B0) {
-        if (fast) {
-          // the common case: two cells per thread, packed; the pair's
-          // primitives from the tile, then the tile is free for the next block
-          float2 Wc[8];
-          if (!a.last && !a.write_u_all) cells_mx_pair_w(reinterpret_cast<const float*>(sT), tid, Wc);
-          __syncthreads();
-          issue_next(NCELL / 2);
-          const float m = cells_mx_pair(a, G, B, blk, Wc, sF, tid, 0.5f * idx0, 0.5f * idx1, 0.5f * idx2, idx0,
-                                        idx1, idx2, gamma);
-          if (a.last) {
-            float mm = m;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-            if ((tid & 31) == 0) sred[tid >> 5] = mm;
-            __syncthreads();
-            if (tid == 0) {
-              float mx = 0.f;
-              for (int w = 0; w < STAGE_THREADS / 32; w++) mx = fmaxf(mx, sred[w]);
-              const double md = f2d_int(mx);
-              if (md > 0.0) atomicMax(&a.smax_next[B.grid], static_cast<unsigned long long>(__double_as_longlong(md)));
-            }
-          }
-          __syncthreads();
-          continue;
-        }
-      }
       auto run_cells = [&](const bool commit) -> bool {
         return fast ? cells(commit, std::true_type{}) : cells(commit, std::false_type{});
       };
@@ -2633,7 +2915,6 @@ __global__ void __launch_bounds__(StageCfg<MIXED>::THREADS, (MIXED && !LRN) ? 2 
       }
       run_cells(true);
       __syncthreads();
-      issue_next(0);
     }
     if (mfail) break;
   }
