@@ -23,12 +23,12 @@ namespace batsk {
 size_t stage_smem_bytes(bool mixed);
 cudaError_t stage_setup(int occ[2]);
 cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const StageArgs& a);
-cudaError_t launch_to_internal(const double* ext, double* in, int block0, int nb, cudaStream_t st);
-cudaError_t launch_to_external(const double* in, double* ext, int block0, int nb, cudaStream_t st);
+cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,
+                              const BlockDev* blocks, const PhysDev& ph, int b0, int nb, unsigned long long* smax,
+                              cudaStream_t st);
+cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, const GridDev* grids,
+                               const BlockDev* blocks, int b0, int nb, cudaStream_t st);
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st);
-cudaError_t launch_prim_mixed(const double* U, float* Wt, int b0, int nb, float gm1f, cudaStream_t st);
-cudaError_t launch_cfl(bool mixed, const double* U, const float* Wt, const GridDev* grids, const BlockDev* blocks,
-                       const PhysDev& ph, int b0, int nb, unsigned long long* smax, cudaStream_t st);
 cudaError_t launch_amr_ghosts(const StageArgs& a, const GhostTask* tasks, const int32_t* gtab, int ntasks,
                               cudaStream_t st);
 cudaError_t launch_amr_ghost_table(const StageArgs& a, const GhostTask* tasks, int32_t* gtab, int ntasks,
@@ -540,14 +540,23 @@ int launch_stage(bats_t* h, const StageArgs& a) {
   return launch_stage_one(h, u, false);  // same stage input: the ghost slabs are in place
 }
 
-// CFL bound of grid g's current state into smax[g]; with dtc, also every
-// cell's local dt = cfl / s_i.
-int launch_cfl(bats_t* h, int g, double* dtc = nullptr, double cfl = 0.0) {
-  const GridDev& G = h->grids_h[g];
-  CK(h, cudaMemsetAsync(h->smax + g, 0, sizeof(unsigned long long), h->stream));
+// The caller's state of blocks [b0, b0 + nb) (ext_off as in k_load_state) into the
+// handle, with the mixed form's primitives and the grids' CFL bounds.
+int load_state(bats_t* h, const double* ext, int64_t ext_off, int g0, int ng, int b0, int nb) {
+  CK(h, cudaMemsetAsync(h->smax + g0, 0, sizeof(unsigned long long) * ng, h->stream));
+  CK(h, launch_load_state(h->ph.precision == BATS_MIXED, ext, ext_off, h->U, h->W, h->grids_d, h->blocks_d, h->ph, b0,
+                          nb, h->smax, h->stream));
+  CK(h, cudaMemsetAsync(h->t + g0, 0, sizeof(double) * ng, h->stream));
+  return BATS_OK;
+}
+
+// CFL bounds of the current states into smax and every cell's local dt = cfl / s_i
+// into dtc.
+int launch_local_dt(bats_t* h, double* dtc, double cfl) {
+  CK(h, cudaMemsetAsync(h->smax, 0, sizeof(unsigned long long) * h->ngrids, h->stream));
   h->launches++;
-  CK(h, launch_cfl_dt(h->ph.precision == BATS_MIXED, h->U, h->W, h->grids_d, h->blocks_d, h->ph, G.block0, G.nb,
-                      h->smax, dtc, cfl, h->stream));
+  CK(h, launch_cfl_dt(h->ph.precision == BATS_MIXED, h->U, h->W, h->grids_d, h->blocks_d, h->ph, 0, h->nbt, h->smax,
+                      dtc, cfl, h->stream));
   return BATS_OK;
 }
 
@@ -584,10 +593,8 @@ int enqueue_steps(bats_t* h, int n, double cfl, double fixed_dt, bool timed, boo
   if (lts && n > 0) {
     // every cell's dt from the current state (later steps take it from the
     // last stage of the step before)
-    for (int g = 0; g < h->ngrids; g++) {
-      int rc = launch_cfl(h, g, h->dtc, cfl);
-      if (rc) return rc;
-    }
+    int rc = launch_local_dt(h, h->dtc, cfl);
+    if (rc) return rc;
   }
   // the one-stage scheme cannot write in place (other blocks read this
   // block's cells as ghosts): it alternates between the two state buffers
@@ -950,12 +957,8 @@ int bats_set_state(bats_t* h, int grid, const double* U, size_t n) {
     CK(h, cudaMemcpyAsync(h->staging, U, need * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     src = h->staging;
   }
-  CK(h, launch_to_internal(src, h->U, G.block0, G.nb, h->stream));
-  if (h->ph.precision == BATS_MIXED)
-    CK(h, launch_prim_mixed(h->U, h->W, G.block0, G.nb, static_cast<float>(h->ph.gm1), h->stream));
-  rc = launch_cfl(h, grid);
+  rc = load_state(h, src, -static_cast<int64_t>(G.block0) * NV * NCELL, grid, 1, G.block0, G.nb);
   if (rc) return rc;
-  CK(h, cudaMemsetAsync(h->t + grid, 0, sizeof(double), h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   return BATS_OK;
 }
@@ -968,7 +971,8 @@ int bats_get_state(bats_t* h, int grid, double* U, size_t n) {
   if (!U || n != need) return fail(h, BATS_ERR_INVALID_ARG, "state size mismatch: expected " + std::to_string(need));
   bool dev = is_device_ptr(U);
   double* dst = dev ? U : h->staging;
-  CK(h, launch_to_external(h->U, dst, G.block0, G.nb, h->stream));
+  CK(h, launch_store_state(h->U, dst, -static_cast<int64_t>(G.block0) * NV * NCELL, h->grids_d, h->blocks_d, G.block0,
+                           G.nb, h->stream));
   if (!dev) CK(h, cudaMemcpyAsync(U, h->staging, need * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   return BATS_OK;
@@ -991,17 +995,7 @@ int bats_set_states(bats_t* h, const double* U, size_t n) {
       src = h->U1;
     }
   }
-  for (int g = 0; g < h->ngrids; g++) {
-    const GridDev& G = h->grids_h[g];
-    CK(h, launch_to_internal(src + static_cast<size_t>(G.block0) * NV * NCELL, h->U, G.block0, G.nb, h->stream));
-  }
-  if (h->ph.precision == BATS_MIXED)
-    CK(h, launch_prim_mixed(h->U, h->W, 0, h->nbt, static_cast<float>(h->ph.gm1), h->stream));
-  for (int g = 0; g < h->ngrids; g++) {
-    int rc = launch_cfl(h, g);
-    if (rc) return rc;
-  }
-  CK(h, cudaMemsetAsync(h->t, 0, sizeof(double) * h->ngrids, h->stream));
+  if (int rc = load_state(h, src, 0, 0, h->ngrids, 0, h->nbt)) return rc;
   CK(h, cudaStreamSynchronize(h->stream));
   return BATS_OK;
 }
@@ -1013,10 +1007,7 @@ int bats_get_states(bats_t* h, double* U, size_t n) {
   const bool dev = is_device_ptr(U);
   double* pinned = dev ? nullptr : static_cast<double*>(const_cast<void*>(device_view_of_pinned(U)));
   double* dst = dev ? U : (pinned ? pinned : h->U1);
-  for (int g = 0; g < h->ngrids; g++) {
-    const GridDev& G = h->grids_h[g];
-    CK(h, launch_to_external(h->U, dst + static_cast<size_t>(G.block0) * NV * NCELL, G.block0, G.nb, h->stream));
-  }
+  CK(h, launch_store_state(h->U, dst, 0, h->grids_d, h->blocks_d, 0, h->nbt, h->stream));
   if (!dev && !pinned) CK(h, cudaMemcpyAsync(U, h->U1, need * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   return BATS_OK;
@@ -1131,7 +1122,8 @@ int bats_debug_residual(bats_t* h, int grid, double* R, size_t n) {
   if (rc) return rc;
   bool dev = is_device_ptr(R);
   double* dst = dev ? R : h->staging;
-  CK(h, launch_to_external(h->U1, dst, G.block0, G.nb, h->stream));
+  CK(h, launch_store_state(h->U1, dst, -static_cast<int64_t>(G.block0) * NV * NCELL, h->grids_d, h->blocks_d, G.block0,
+                           G.nb, h->stream));
   if (!dev) CK(h, cudaMemcpyAsync(R, h->staging, need * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   return index_check(h);

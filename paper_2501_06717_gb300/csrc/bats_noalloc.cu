@@ -9,8 +9,8 @@
 // allocated per call, on the device or on the host heap: the grid tables are
 // built in fixed-capacity arrays on the caller's stack (about 80 KB).
 //
-// The kernels are the ones bats_step uses (k_stage FP64 form, k_cfl, k_dt and
-// the layout transposes); only where their scratch lives differs.
+// The kernels are the ones bats_step uses (k_stage FP64 form, k_load_state, k_dt
+// and k_store_state); only where their scratch lives differs.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -26,11 +26,12 @@ namespace batsk {
 size_t stage_smem_bytes(bool mixed);
 cudaError_t stage_setup(int occ[2]);
 cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const StageArgs& a);
-cudaError_t launch_to_internal(const double* ext, double* in, int block0, int nb, cudaStream_t st);
-cudaError_t launch_to_external(const double* in, double* ext, int block0, int nb, cudaStream_t st);
+cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,
+                              const BlockDev* blocks, const PhysDev& ph, int b0, int nb, unsigned long long* smax,
+                              cudaStream_t st);
+cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, const GridDev* grids,
+                               const BlockDev* blocks, int b0, int nb, cudaStream_t st);
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st);
-cudaError_t launch_cfl(bool mixed, const double* U, const float* Wt, const GridDev* grids, const BlockDev* blocks,
-                       const PhysDev& ph, int b0, int nb, unsigned long long* smax, cudaStream_t st);
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
                       unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st);
 cudaError_t read_index_flag(int32_t* out);
@@ -357,8 +358,7 @@ extern "C" int bats_step_noalloc(const bats_grid_desc* grid, const bats_physics*
   const bool dev_ptr = device_pointer(U);
   const size_t bytes = n * sizeof(double);
   if (!dev_ptr) NA_CK(cudaMemcpyAsync(U1, U, bytes, cudaMemcpyHostToDevice, st));
-  NA_CK(launch_to_internal(dev_ptr ? U : U1, Ui, 0, nb, st));
-  NA_CK(launch_cfl(false, Ui, nullptr, G, blocks, ph, 0, nb, smax, st));
+  NA_CK(launch_load_state(false, dev_ptr ? U : U1, 0, Ui, nullptr, G, blocks, ph, 0, nb, smax, st));
 
   const bool ssp = ph.rk == BATS_RK_SSP2;
   const bool euler = ph.rk == BATS_RK_EULER;
@@ -412,7 +412,7 @@ extern "C" int bats_step_noalloc(const bats_grid_desc* grid, const bats_physics*
   }
   if (Ucur != Ui) NA_CK(cudaMemcpyAsync(Ui, Ucur, bytes, cudaMemcpyDeviceToDevice, st));
   // block-major -> caller layout (host destinations staged through U1)
-  NA_CK(launch_to_external(Ui, dev_ptr ? U : U1, 0, nb, st));
+  NA_CK(launch_store_state(Ui, dev_ptr ? U : U1, 0, G, blocks, 0, nb, st));
   if (!dev_ptr) NA_CK(cudaMemcpyAsync(U, U1, bytes, cudaMemcpyDeviceToHost, st));
   int32_t ew[3];
   double tt = 0.0;

@@ -135,30 +135,6 @@ __global__ void __launch_bounds__(128) k_amr_ghosts(const StageArgs a, const Gho
 // ---------------------------------------------------------------------------
 // Small kernels.
 
-// [8][nb][512] (external) <-> [nb][8][512] (internal) for blocks block0..block0+nb
-__global__ void k_to_internal(const double* __restrict__ ext, double* __restrict__ in, int block0, int nb) {
-  int64_t n = static_cast<int64_t>(nb) * NV * NCELL;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int c = static_cast<int>(e % NCELL);
-    int64_t r = e / NCELL;
-    int b = static_cast<int>(r % nb);
-    int v = static_cast<int>(r / nb);
-    in[(static_cast<int64_t>(block0 + b) * NV + v) * NCELL + c] = ext[e];
-  }
-}
-__global__ void k_to_external(const double* __restrict__ in, double* __restrict__ ext, int block0, int nb) {
-  int64_t n = static_cast<int64_t>(nb) * NV * NCELL;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int c = static_cast<int>(e % NCELL);
-    int64_t r = e / NCELL;
-    int b = static_cast<int>(r % nb);
-    int v = static_cast<int>(r / nb);
-    ext[e] = in[(static_cast<int64_t>(block0 + b) * NV + v) * NCELL + c];
-  }
-}
-
 // Conservative inflow/body states (and the mixed-form primitives of the inflow).
 __global__ void k_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1) {
   int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -171,70 +147,140 @@ __global__ void k_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, d
   for (int v = 0; v < NV; v++) G.Winflow32[v] = w[v];
 }
 
-// Mixed form: W = FP32 primitives of U for blocks [b0, b0+nb).
-__global__ void k_prim_mixed(const double* __restrict__ U, float* __restrict__ Wt, int b0, int nb, float gm1f) {
-  int64_t n = static_cast<int64_t>(nb) * NCELL;
-  for (int64_t e = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    int blk = b0 + static_cast<int>(e / NCELL), c = static_cast<int>(e % NCELL);
-    int64_t base = static_cast<int64_t>(blk) * NV * NCELL + c;
-    double u[8];
-    float w[8];
-    for (int v = 0; v < NV; v++) u[v] = U[base + v * NCELL];
-    prim_mixed(u, gm1f, w);
-    for (int v = 0; v < NV; v++) Wt[base + v * NCELL] = w[v];
+// CFL bound sum_d (|u_d| + c_f,d) / dx_d of cell c of block B (-1 in the body)
+// from its FP32 primitives (mixed form) or its conservative state.
+__device__ __forceinline__ double cfl_cell(const GridDev& G, const BlockDev& B, const PhysDev& ph, int c, const float* W,
+                                           const double* U) {
+  double xc[3] = {0.0, 0.0, 0.0};
+  if (G.body_r > 0.0 || ph.b0 != B0_NONE) {
+    const int ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6;
+    xc[0] = G.lo[0] + ((static_cast<double>(B.bi * NC) + ci) + 0.5) * G.dx[B.level][0];
+    xc[1] = G.lo[1] + ((static_cast<double>(B.bj * NC) + cj) + 0.5) * G.dx[B.level][1];
+    xc[2] = G.lo[2] + ((static_cast<double>(B.bk * NC) + ck) + 0.5) * G.dx[B.level][2];
+    if (G.body_r > 0.0 && (xc[0] * xc[0] + xc[1] * xc[1] + xc[2] * xc[2]) < G.body_r * G.body_r) return -1.0;
+  }
+  if (W) {
+    float B0c[3] = {0.f, 0.f, 0.f};
+    const float xr[3] = {float(xc[0]), float(xc[1]), float(xc[2])};
+    if (ph.b0 != B0_NONE) b0_at<float>(ph, xr, B0c);
+    const float Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
+    float sf = 0.f;
+#pragma unroll
+    for (int e = 0; e < 3; e++) {
+      const float cf = fast_speed_n(ph.gammaf, W[0], W[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
+      sf = sf + (fabsf(W[1 + e]) + cf) * rcp_approx(G.dxf[B.level][e]);
+    }
+    return f2d_int(sf);
+  }
+  double V[8], B0c[3] = {0.0, 0.0, 0.0};
+  prim64(U, ph.gm1, V);
+  if (ph.b0 != B0_NONE) b0_at<double>(ph, xc, B0c);
+  const double Bt[3] = {B0c[0] + V[4], B0c[1] + V[5], B0c[2] + V[6]};
+  return cfl_sum64(ph.gamma, V, Bt, G.idx[B.level]);
+}
+// The largest of the CTA's bounds into smax of its grid (a NaN counts as none).
+__device__ __forceinline__ void cfl_reduce(double s, unsigned long long* smax) {
+  __shared__ unsigned long long sred[16];
+  unsigned long long m = s > 0.0 ? static_cast<unsigned long long>(__double_as_longlong(s)) : 0ull;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long q = __shfl_xor_sync(0xffffffffu, m, o);
+    m = q > m ? q : m;
+  }
+  if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < static_cast<int>(blockDim.x) / 32; w++) m = sred[w] > m ? sred[w] : m;
+    if (m) atomicMax(smax, m);
   }
 }
 
-// CFL bound of the current state for blocks [b0, b0+nb): one CTA per block.
+// Loading a state: one CTA of 256 threads per block, cells t and t + 256 per
+// thread.  ext [8][nb][512] per grid, grid after grid (element (v, b, c) of a
+// grid at ext_off + 4096 block0 + (v nb + b) 512 + c) -> U [block][8][512], the
+// mixed form's primitives and the CFL bound, in one pass and one launch for all
+// grids: bound by memory (128 bytes per cell, 160 in the mixed form; 8 grids, 3.1
+// M cells, mixed: 74 us, 6.0 TB/s).  Launches per grid for the layout (64-bit
+// divisions per element), the primitives and the bound, and for the way back,
+// took 6.6 ms for 64 grids (30 M cells), one launch each way 1.3 ms.
 template <bool MIXED>
-__global__ void k_cfl(const double* __restrict__ U, const float* __restrict__ Wt, const GridDev* grids,
-                      const BlockDev* blocks, PhysDev ph, int b0, unsigned long long* smax, double* dtc, double cfl) {
-  __shared__ double sred[NCELL / 32];
-  int blk = b0 + blockIdx.x, c = threadIdx.x;
-  const BlockDev B = blocks[blk];
+__global__ void __launch_bounds__(256) k_load_state(const double* __restrict__ ext, int64_t ext_off,
+                                                    double* __restrict__ U, float* __restrict__ Wt,
+                                                    const GridDev* __restrict__ grids,
+                                                    const BlockDev* __restrict__ blocks, const PhysDev ph, int b0,
+                                                    unsigned long long* smax) {
+  const int blk = b0 + blockIdx.x;
+  const BlockDev& B = blocks[blk];
   const GridDev& G = grids[B.grid];
-  int ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6;
-  double dxd[3], xc[3];
-  for (int d = 0; d < 3; d++) dxd[d] = (G.hi[d] - G.lo[d]) / static_cast<double>((static_cast<int64_t>(G.root[d]) << B.level) * NC);
-  xc[0] = G.lo[0] + ((static_cast<double>(B.bi * NC) + ci) + 0.5) * dxd[0];
-  xc[1] = G.lo[1] + ((static_cast<double>(B.bj * NC) + cj) + 0.5) * dxd[1];
-  xc[2] = G.lo[2] + ((static_cast<double>(B.bk * NC) + ck) + 0.5) * dxd[2];
-  bool in_body = G.body_r > 0.0 && (xc[0] * xc[0] + xc[1] * xc[1] + xc[2] * xc[2]) < G.body_r * G.body_r;
-  int64_t base = static_cast<int64_t>(blk) * NV * NCELL + c;
+  const int64_t vstride = static_cast<int64_t>(G.nb) * NCELL;
+  const double* src = ext + ext_off + static_cast<int64_t>(G.block0) * (NV * NCELL) +
+                      static_cast<int64_t>(blk - G.block0) * NCELL;
+  const int64_t base = static_cast<int64_t>(blk) * (NV * NCELL);
+  double u[2][8];
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    u[0][v] = src[v * vstride + threadIdx.x];
+    u[1][v] = src[v * vstride + threadIdx.x + 256];
+  }
   double s = 0.0;
-  if (!in_body) {
+#pragma unroll
+  for (int h = 0; h < 2; h++) {
+    const int c = threadIdx.x + 256 * h;
+    float w[8];
+#pragma unroll
+    for (int v = 0; v < NV; v++) U[base + v * NCELL + c] = u[h][v];
     if constexpr (MIXED) {
-      float W[8], B0c[3] = {0.f, 0.f, 0.f};
-      for (int v = 0; v < NV; v++) W[v] = Wt[base + v * NCELL];
-      float xr[3] = {float(xc[0]), float(xc[1]), float(xc[2])};
-      if (ph.b0 != B0_NONE) b0_at<float>(ph, xr, B0c);
-      float Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
-      float sf = 0.f;
-      for (int e = 0; e < 3; e++) {
-        float cf = fast_speed_n(float(ph.gamma), W[0], W[7], Bt[e], Bt[(e + 1) % 3], Bt[(e + 2) % 3]);
-        sf = sf + (fabsf(W[1 + e]) + cf) * rcp_approx(float(dxd[e]));
-      }
-      s = sf;
-    } else {
-      double u[8], W[8], B0c[3] = {0, 0, 0};
-      for (int v = 0; v < NV; v++) u[v] = U[base + v * NCELL];
-      prim64(u, ph.gm1, W);
-      if (ph.b0 != B0_NONE) b0_at<double>(ph, xc, B0c);
-      const double Bt[3] = {B0c[0] + W[4], B0c[1] + W[5], B0c[2] + W[6]};
-      s = cfl_sum64(ph.gamma, W, Bt, G.idx[B.level]);
+      prim_mixed(u[h], ph.gm1f, w);
+#pragma unroll
+      for (int v = 0; v < NV; v++) Wt[base + v * NCELL + c] = w[v];
     }
+    const double q = cfl_cell(G, B, ph, c, MIXED ? w : nullptr, u[h]);
+    s = q > s ? q : s;
   }
-  // local time stepping: the cell's own dt (0 in the body)
-  if (dtc) dtc[static_cast<int64_t>(blk) * NCELL + c] = in_body ? 0.0 : cfl / s;
-  for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
-  if ((c & 31) == 0) sred[c >> 5] = s;
-  __syncthreads();
-  if (c == 0) {
-    double m = 0.0;
-    for (int w = 0; w < NCELL / 32; w++) m = fmax(m, sred[w]);
-    if (m > 0.0) atomicMax(&smax[B.grid], static_cast<unsigned long long>(__double_as_longlong(m)));
+  cfl_reduce(s, &smax[B.grid]);
+}
+// The way back, blocks [b0, b0 + gridDim.x).
+__global__ void __launch_bounds__(256) k_store_state(const double* __restrict__ U, double* __restrict__ ext,
+                                                     int64_t ext_off, const GridDev* __restrict__ grids,
+                                                     const BlockDev* __restrict__ blocks, int b0) {
+  const int blk = b0 + blockIdx.x;
+  const GridDev& G = grids[blocks[blk].grid];
+  const int64_t vstride = static_cast<int64_t>(G.nb) * NCELL;
+  double* dst = ext + ext_off + static_cast<int64_t>(G.block0) * (NV * NCELL) +
+                static_cast<int64_t>(blk - G.block0) * NCELL + threadIdx.x;
+  const double* src = U + static_cast<int64_t>(blk) * (NV * NCELL) + threadIdx.x;
+  double u[16];
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    u[2 * v] = src[v * NCELL];
+    u[2 * v + 1] = src[v * NCELL + 256];
   }
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    dst[v * vstride] = u[2 * v];
+    dst[v * vstride + 256] = u[2 * v + 1];
+  }
+}
+
+// CFL bound of the current state and, with dtc, every cell's local dt (0 in the
+// body): one CTA per block.
+template <bool MIXED>
+__global__ void __launch_bounds__(NCELL) k_cfl(const double* __restrict__ U, const float* __restrict__ Wt,
+                                               const GridDev* grids, const BlockDev* blocks, const PhysDev ph, int b0,
+                                               unsigned long long* smax, double* dtc, double cfl) {
+  const int blk = b0 + blockIdx.x, c = threadIdx.x;
+  const BlockDev& B = blocks[blk];
+  const int64_t base = static_cast<int64_t>(blk) * NV * NCELL + c;
+  double u[8], s;
+  float w[8];
+#pragma unroll
+  for (int v = 0; v < NV; v++) {
+    if constexpr (MIXED) w[v] = Wt[base + v * NCELL];
+    else u[v] = U[base + v * NCELL];
+  }
+  s = cfl_cell(grids[B.grid], B, ph, c, MIXED ? w : nullptr, u);
+  if (dtc) dtc[static_cast<int64_t>(blk) * NCELL + c] = s < 0.0 ? 0.0 : cfl / s;
+  cfl_reduce(s, &smax[B.grid]);
 }
 
 // Refluxing after a stage.  One CTA per corrected block, one thread per face
@@ -586,22 +632,20 @@ cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const Sta
   return cudaGetLastError();
 }
 
-static int grid_for(int64_t n) { return static_cast<int>(std::min<int64_t>((n + 255) / 256, 4096)); }
-
-cudaError_t launch_to_internal(const double* ext, double* in, int block0, int nb, cudaStream_t st) {
-  k_to_internal<<<grid_for(static_cast<int64_t>(nb) * NV * NCELL), 256, 0, st>>>(ext, in, block0, nb);
+cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,
+                              const BlockDev* blocks, const PhysDev& ph, int b0, int nb, unsigned long long* smax,
+                              cudaStream_t st) {
+  if (mixed) k_load_state<true><<<nb, 256, 0, st>>>(ext, ext_off, U, W, grids, blocks, ph, b0, smax);
+  else k_load_state<false><<<nb, 256, 0, st>>>(ext, ext_off, U, W, grids, blocks, ph, b0, smax);
   return cudaGetLastError();
 }
-cudaError_t launch_to_external(const double* in, double* ext, int block0, int nb, cudaStream_t st) {
-  k_to_external<<<grid_for(static_cast<int64_t>(nb) * NV * NCELL), 256, 0, st>>>(in, ext, block0, nb);
+cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, const GridDev* grids,
+                               const BlockDev* blocks, int b0, int nb, cudaStream_t st) {
+  k_store_state<<<nb, 256, 0, st>>>(U, ext, ext_off, grids, blocks, b0);
   return cudaGetLastError();
 }
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st) {
   k_init_grid_states<<<(ngrids + 63) / 64, 64, 0, st>>>(grids, ngrids, inv_gm1, gm1);
-  return cudaGetLastError();
-}
-cudaError_t launch_prim_mixed(const double* U, float* Wt, int b0, int nb, float gm1f, cudaStream_t st) {
-  k_prim_mixed<<<grid_for(static_cast<int64_t>(nb) * NCELL), 256, 0, st>>>(U, Wt, b0, nb, gm1f);
   return cudaGetLastError();
 }
 cudaError_t launch_cfl_dt(bool mixed, const double* U, const float* Wt, const GridDev* grids,
@@ -629,10 +673,6 @@ cudaError_t launch_reflux(bool mixed, const StageArgs& a, const RefluxTask* task
   if (mixed) k_reflux<true><<<nrb, 64, 0, st>>>(a, tasks, rblocks);
   else k_reflux<false><<<nrb, 64, 0, st>>>(a, tasks, rblocks);
   return cudaGetLastError();
-}
-cudaError_t launch_cfl(bool mixed, const double* U, const float* Wt, const GridDev* grids, const BlockDev* blocks,
-                       const PhysDev& ph, int b0, int nb, unsigned long long* smax, cudaStream_t st) {
-  return launch_cfl_dt(mixed, U, Wt, grids, blocks, ph, b0, nb, smax, nullptr, 0.0, st);
 }
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
                       unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st) {
