@@ -560,7 +560,9 @@ int launch_local_dt(bats_t* h, double* dtc, double cfl) {
   return BATS_OK;
 }
 
-constexpr int kMaxTimedSteps = 256;
+// Timed steps of a call: an event node between two kernels of a graph costs about
+// 4 us, so all 100 steps of 120 blocks took 4.0 ms with theirs and 3.0 ms without.
+constexpr int kMaxTimedSteps = 8;
 
 int ensure_stage_events(bats_t* h, int n) {
   int want = 2 * std::min(n, kMaxTimedSteps);
@@ -724,6 +726,7 @@ int run_steps(bats_t* h, int n, double cfl, double fixed_dt, double* t_out) {
     stage_ms += m;
   }
   if (h->timed_steps > 0 && n > h->timed_steps) stage_ms *= static_cast<double>(n) / h->timed_steps;
+  stage_ms = std::min(stage_ms, static_cast<double>(ms));  // (scaled from the first steps)
   h->ms_last[BATS_PHASE_STAGE] = h->timed_steps > 0 ? stage_ms : -1.0;
   h->ms_last[BATS_PHASE_DT] = h->timed_steps > 0 ? ms - stage_ms : -1.0;
   h->ms_last[BATS_PHASE_TOTAL] = ms;

@@ -96,9 +96,11 @@ __global__ void __launch_bounds__(128) k_amr_ghosts(const StageArgs a, const Gho
   const int32_t ent = gtab[static_cast<int64_t>(blockIdx.x) * 128 + tid];
   const BlockDev& B = a.blocks[chki(T.blk, 0, a.nblocks)];
   const GridDev& G = a.grids[B.grid];
+  const bool coarser = B.ftype[T.s] == FACE_COARSER;
+  pdl_begin();  // the tables above are static
   float w[8];
   int g[3];
-  if (B.ftype[T.s] == FACE_COARSER) {
+  if (coarser) {
     if (ent != GT_NONE) {
       const int lev = ghost_sample(T, B, tid, g);
       float ws[8], u[8];
@@ -439,6 +441,7 @@ __global__ void __launch_bounds__(64) k_reflux(const StageArgs a, const RefluxTa
 //  mode 1 (after a step):  t += dt; smax = smax_next
 __global__ void k_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
                      unsigned long long* smax, unsigned long long* smax_next) {
+  pdl_begin();
   int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= ngrids) return;
   if (mode == 0) {
@@ -565,6 +568,22 @@ static size_t stage_smem(bool mixed, bool lrn) {
   return mixed ? (lrn ? kSmemLx : StageCfg<true>::SMEM_MX) : StageCfg<false>::SMEM;
 }
 
+// Launch of a kernel that begins with pdl_wait or pdl_begin.
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, args...);
+}
+
 using StageFn = void (*)(const StageArgs);
 template <bool MIXED, bool LRN, int FLX>
 StageFn stage_fn_l(int lim, bool b0) {
@@ -626,10 +645,9 @@ cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const Sta
   const bool lrn = a.learned || a.kind >= 3;
   const int flux = a.ph.flux;
   if (mixed)
-    stage_fn<true>(a.ph.limiter, b0, lrn, flux)<<<grid, lrn ? STAGE_THREADS : MX_THREADS, stage_smem(true, lrn), st>>>(a);
-  else
-    stage_fn<false>(a.ph.limiter, b0, lrn, flux)<<<grid, STAGE_THREADS, StageCfg<false>::SMEM, st>>>(a);
-  return cudaGetLastError();
+    return launch_pdl(stage_fn<true>(a.ph.limiter, b0, lrn, flux), grid, lrn ? STAGE_THREADS : MX_THREADS,
+                      stage_smem(true, lrn), st, a);
+  return launch_pdl(stage_fn<false>(a.ph.limiter, b0, lrn, flux), grid, STAGE_THREADS, StageCfg<false>::SMEM, st, a);
 }
 
 cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,
@@ -664,8 +682,7 @@ cudaError_t launch_amr_ghost_table(const StageArgs& a, const GhostTask* tasks, i
 cudaError_t launch_amr_ghosts(const StageArgs& a, const GhostTask* tasks, const int32_t* gtab, int ntasks,
                               cudaStream_t st) {
   if (ntasks <= 0) return cudaSuccess;
-  k_amr_ghosts<<<ntasks, 128, 0, st>>>(a, tasks, gtab);
-  return cudaGetLastError();
+  return launch_pdl(k_amr_ghosts, ntasks, 128, 0, st, a, tasks, gtab);
 }
 cudaError_t launch_reflux(bool mixed, const StageArgs& a, const RefluxTask* tasks, const int32_t* rblocks, int nrb,
                           cudaStream_t st) {
@@ -676,8 +693,7 @@ cudaError_t launch_reflux(bool mixed, const StageArgs& a, const RefluxTask* task
 }
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
                       unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st) {
-  k_dt<<<(ngrids + 127) / 128, 128, 0, st>>>(ngrids, mode, cfl, fixed_dt, dt, t, smax, smax_next);
-  return cudaGetLastError();
+  return launch_pdl(k_dt, (ngrids + 127) / 128, 128, 0, st, ngrids, mode, cfl, fixed_dt, dt, t, smax, smax_next);
 }
 cudaError_t launch_debug_fill(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st) {
   k_debug_fill<<<nb, 256, sizeof(double) * (NV * NTILE + 3 * 128 * NV), st>>>(a, b0, nb, T);
