@@ -285,7 +285,7 @@ int build_grid(bats_t* h, const bats_grid_desc& d, int gidx, int block0, std::ve
     for (int f = 0; f < 6; f++)
       if (B.ftype[f] == FACE_COARSER || B.ftype[f] == FACE_FINER) {
         B.rslot[f] = h->nslots++;
-        h->gtasks_h.push_back(GhostTask{block0 + b, f, B.rslot[f]});
+        h->gtasks_h.push_back(GhostTask{block0 + b, f, B.rslot[f], B.ftype[f] == FACE_COARSER});
       }
   }
   for (int b = 0; b < d.n_leaves; b++) {

@@ -104,8 +104,9 @@ struct RefluxTask {
 // Mixed form: one face of a block at a resolution change (COARSER or FINER),
 // whose face-slab ghosts are computed ahead of the stage into slot `slot` of
 // the ghost-slab buffer.
-struct GhostTask {
+struct alignas(16) GhostTask {
   int32_t blk, s, slot;
+  int32_t coarser;  // the neighbour is coarser (prolongation), else finer (restriction)
 };
 
 // Arguments of one stage launch.

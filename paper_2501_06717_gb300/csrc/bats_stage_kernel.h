@@ -698,36 +698,39 @@ __device__ __forceinline__ float sum8(const float c[8]) {
 // at p (a leaf's FP32 primitives, variable stride NCELL) to one coarse cell,
 // as primitives: density and field the means, velocity the mass-weighted
 // mean, pressure the mean plus the velocity and field variances.
-static __device__ __noinline__ void restrict_at(const float* p, float gm1f, float w[8]) {
-  const int off[8] = {0, 1, NC, NC + 1, NC * NC, NC * NC + 1, NC * NC + NC, NC * NC + NC + 1};
-  float rho[8], c[8];
+// (All 64 loads are issued before the first use: one latency instead of eight.)
+__device__ __forceinline__ void restrict_at(const float* p, float gm1f, float w[8]) {
+  float x[8][8];  // [variable][child: i, j, k bits]; the corner cell is even along i: 8-byte pairs
 #pragma unroll
-  for (int o = 0; o < 8; o++) rho[o] = p[off[o]];
-  const float srho = sum8(rho);
+  for (int v = 0; v < NV; v++)
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+      const float2 q = *reinterpret_cast<const float2*>(p + v * NCELL + (r & 1) * NC + (r >> 1) * NC * NC);
+      x[v][2 * r] = q.x;
+      x[v][2 * r + 1] = q.y;
+    }
+  float c[8];
+  const float srho = sum8(x[0]);
   const float irs = rcp_approx(srho);
   float ut[3], var = 0.f;
 #pragma unroll
   for (int e = 0; e < 3; e++) {
-    float u[8];
-#pragma unroll
-    for (int o = 0; o < 8; o++) u[o] = p[(1 + e) * NCELL + off[o]];
+    const float* u = x[1 + e];
     const float ub = 0.125f * sum8(u);
 #pragma unroll
-    for (int o = 0; o < 8; o++) c[o] = rho[o] * (u[o] - ub);
+    for (int o = 0; o < 8; o++) c[o] = x[0][o] * (u[o] - ub);
     ut[e] = ub + sum8(c) * irs;
 #pragma unroll
     for (int o = 0; o < 8; o++) {
       const float du = u[o] - ut[e];
-      c[o] = rho[o] * du * du;
+      c[o] = x[0][o] * du * du;
     }
     var += sum8(c);
   }
   float bt[3];
 #pragma unroll
   for (int e = 0; e < 3; e++) {
-    float b[8];
-#pragma unroll
-    for (int o = 0; o < 8; o++) b[o] = p[(4 + e) * NCELL + off[o]];
+    const float* b = x[4 + e];
     bt[e] = 0.125f * sum8(b);
 #pragma unroll
     for (int o = 0; o < 8; o++) {
@@ -736,8 +739,6 @@ static __device__ __noinline__ void restrict_at(const float* p, float gm1f, floa
     }
     var += sum8(c);
   }
-#pragma unroll
-  for (int o = 0; o < 8; o++) c[o] = p[7 * NCELL + off[o]];
   w[0] = 0.125f * srho;
   w[1] = ut[0];
   w[2] = ut[1];
@@ -745,7 +746,7 @@ static __device__ __noinline__ void restrict_at(const float* p, float gm1f, floa
   w[4] = bt[0];
   w[5] = bt[1];
   w[6] = bt[2];
-  w[7] = 0.125f * sum8(c) + gm1f * (0.0625f * var);
+  w[7] = 0.125f * sum8(x[7]) + gm1f * (0.0625f * var);
 }
 
 static __device__ __noinline__ void restrict_w(const float* Wt, const GridDev& G, const BlockDev* blocks,
@@ -821,43 +822,40 @@ __device__ __forceinline__ bool psample(const BlockDev& B, int s, int k, int gc[
   return true;
 }
 
-// Fine ghost cell `local` (0..127, as in the face slab) of COARSER face s
-// from the sample table: the coarse value plus (+-1/4) x minmod of the
-// undivided coarse differences of the conservative variables (x, then y,
-// then z), turned into primitives from the coarse cell's own primitives and
+// The limited slopes of the 16 coarse cells of COARSER face s from the sample
+// table, minmod of the undivided coarse differences of the conservative
+// variables, once per coarse cell: thread t (of 128) takes variable t >> 4 of
+// cell t & 15 along all three axes, into sl[(axis * 8 + v) * 16 + cell].
+__device__ __forceinline__ void prolong_slopes_w(const float* tab, int s, int t, float* sl) {
+  const int d = s >> 1, side = s & 1, ta = d == 0 ? 1 : 0;
+  const int cc = t & 15, v = t >> 4, ca = cc & 3, cb = cc >> 2;
+  const int kc = (cb + 1) * 6 + (ca + 1), kin = 36 + cc, kfar = 52 + cc;
+  const float uc = tab[kc * PSTRIDE + v];
+#pragma unroll
+  for (int ax = 0; ax < 3; ax++) {
+    const int km = ax == d ? (side ? kin : kfar) : (ax == ta ? kc - 1 : kc - 6);
+    const int kp = ax == d ? (side ? kfar : kin) : (ax == ta ? kc + 1 : kc + 6);
+    sl[(ax * NV + v) * 16 + cc] = minmod_f(uc - tab[km * PSTRIDE + v], tab[kp * PSTRIDE + v] - uc);
+  }
+}
+// Fine ghost cell `local` (0..127, as in the face slab) of COARSER face s from
+// the sample table and the slopes: the coarse value plus (+-1/4) x slope (x, then
+// y, then z), turned into primitives from the coarse cell's own primitives and
 // the increment (prim_increment).
-__device__ __forceinline__ void prolong_child_w(const float* tab, int s, int local, float gm1f, float w[8]) {
-  const int d = s >> 1, side = s & 1;
-  const int ta = d == 0 ? 1 : 0;
+__device__ __forceinline__ void prolong_child_w(const float* tab, const float* sl, int s, int local, float gm1f,
+                                                float w[8]) {
+  const int d = s >> 1, ta = d == 0 ? 1 : 0;
   const int on = local & 1, taf = (local >> 1) & 7, tbf = local >> 4;
   const int ca = taf >> 1, oa = taf & 1, cb = tbf >> 1, ob = tbf & 1;
-  const int kc = (cb + 1) * 6 + (ca + 1);
-  const int kin = 36 + ca + 4 * cb, kfar = 52 + ca + 4 * cb;
-  const float* Uc = tab + kc * PSTRIDE;
+  const float* Uc = tab + ((cb + 1) * 6 + (ca + 1)) * PSTRIDE;
   float dl[8];
 #pragma unroll
   for (int v = 0; v < NV; v++) dl[v] = 0.f;
 #pragma unroll
   for (int ax = 0; ax < 3; ax++) {
-    int km, kp, odd;
-    if (ax == d) {
-      km = side ? kin : kfar;
-      kp = side ? kfar : kin;
-      odd = on;
-    } else if (ax == ta) {
-      km = kc - 1;
-      kp = kc + 1;
-      odd = oa;
-    } else {
-      km = kc - 6;
-      kp = kc + 6;
-      odd = ob;
-    }
-    const float* Um = tab + km * PSTRIDE;
-    const float* Up = tab + kp * PSTRIDE;
-    const float sg = odd ? 0.25f : -0.25f;
+    const float sg = (ax == d ? on : (ax == ta ? oa : ob)) ? 0.25f : -0.25f;
 #pragma unroll
-    for (int v = 0; v < NV; v++) dl[v] = dl[v] + sg * minmod_f(Uc[v] - Um[v], Up[v] - Uc[v]);
+    for (int v = 0; v < NV; v++) dl[v] = dl[v] + sg * sl[(ax * NV + v) * 16 + ca + 4 * cb];
   }
   const float Wc[8] = {Uc[0], Uc[9], Uc[10], Uc[11], Uc[4], Uc[5], Uc[6], Uc[8]};
   prim_increment(Wc, dl, gm1f, w);
