@@ -28,6 +28,8 @@ cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, do
                               cudaStream_t st);
 cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, const GridDev* grids,
                                const BlockDev* blocks, int b0, int nb, cudaStream_t st);
+cudaError_t launch_b0_table(bool mixed, const GridDev* grids, const BlockDev* blocks, const PhysDev& ph, int nb, void* t,
+                            cudaStream_t st);
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st);
 cudaError_t launch_amr_ghosts(const StageArgs& a, const GhostTask* tasks, const int32_t* gtab, int ntasks,
                               cudaStream_t st);
@@ -79,6 +81,7 @@ struct bats {
   size_t staging_n = 0;
   int persistent = 0, bpc = 1, ctas_per_sm = 0, use_graph = 0;
   int local_dt = 0;
+  char* b0t = nullptr;    // background field per cell [nbt][7][512] (FP32 or FP64)
   double* dtc = nullptr;  // local time stepping: per-cell dt [nbt][512]
   // refluxing
   int reflux = 0, nslots = 0;
@@ -410,6 +413,7 @@ void free_all(bats_t* h) {
   cudaFree(h->W);
   cudaFree(h->W1);
   cudaFree(h->dtc);
+  cudaFree(h->b0t);
   cudaFree(h->freg);
   cudaFree(h->gbuf);
   cudaFree(h->gtasks_d);
@@ -451,6 +455,7 @@ StageArgs base_args(bats_t* h) {
   a.nblocks = h->nbt;
   a.nslots = h->nslots;
   a.blocks_per_item = std::max(1, h->bpc);
+  a.b0t = h->b0t;
   a.ph = h->ph;
   return a;
 }
@@ -888,6 +893,13 @@ int bats_create(const bats_grid_desc* grids, int n_grids, const bats_physics* ph
     delete h;
     return rc;
   }
+  if (h->ph.b0 != BATS_B0_NONE &&
+      (rc = dev_alloc(h, &h->b0t, static_cast<size_t>(h->nbt) * 7 * NCELL * (h->ph.precision == BATS_MIXED ? 4 : 8)))) {
+    free_all(h);
+    g_create_error = h->err;
+    delete h;
+    return rc;
+  }
   if (h->local_dt && (rc = dev_alloc(h, &h->dtc, static_cast<size_t>(h->nbt) * NCELL))) {
     free_all(h);
     g_create_error = h->err;
@@ -922,6 +934,8 @@ int bats_create(const bats_grid_desc* grids, int n_grids, const bats_physics* ph
   if (e == cudaSuccess) e = cudaMemsetAsync(h->smax, 0, sizeof(unsigned long long) * h->ngrids, h->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(h->U, 0, sizeof(double) * nstate, h->stream);
   if (e == cudaSuccess) e = launch_init_grid_states(h->grids_d, h->ngrids, h->ph.inv_gm1, h->ph.gm1, h->stream);
+  if (e == cudaSuccess && h->b0t)
+    e = launch_b0_table(h->ph.precision == BATS_MIXED, h->grids_d, h->blocks_d, h->ph, h->nbt, h->b0t, h->stream);
   // the static tree: where every ghost-slab sample of the pre-pass lies
   if (e == cudaSuccess && h->gtab_d)
     e = launch_amr_ghost_table(base_args(h), h->gtasks_d, h->gtab_d, static_cast<int>(h->gtasks_h.size()), h->stream);

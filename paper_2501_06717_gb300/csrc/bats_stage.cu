@@ -291,6 +291,16 @@ __global__ void __launch_bounds__(NCELL) k_cfl(const double* __restrict__ U, con
   cfl_reduce(s, &smax[B.grid]);
 }
 
+// The background-field table of a handle (b0_cell): one CTA per block.
+template <class R>
+__global__ void __launch_bounds__(NCELL) k_b0_table(const GridDev* grids, const BlockDev* blocks, const PhysDev ph, R* t) {
+  const BlockDev& B = blocks[blockIdx.x];
+  R o[7];
+  b0_cell_eval<R>(ph, grids[B.grid], B, threadIdx.x, o);
+#pragma unroll
+  for (int k = 0; k < 7; k++) t[(static_cast<int64_t>(blockIdx.x) * 7 + k) * NCELL + threadIdx.x] = o[k];
+}
+
 // Refluxing after a stage.  One CTA per corrected block, one thread per face
 // position (q, r) of a refined face: the coarse cell next to it trades its own
 // face flux for the mean of the 4 fine fluxes through the face (summed in the
@@ -666,6 +676,12 @@ cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, do
 cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, const GridDev* grids,
                                const BlockDev* blocks, int b0, int nb, cudaStream_t st) {
   k_store_state<<<nb, 256, 0, st>>>(U, ext, ext_off, grids, blocks, b0);
+  return cudaGetLastError();
+}
+cudaError_t launch_b0_table(bool mixed, const GridDev* grids, const BlockDev* blocks, const PhysDev& ph, int nb, void* t,
+                            cudaStream_t st) {
+  if (mixed) k_b0_table<float><<<nb, NCELL, 0, st>>>(grids, blocks, ph, static_cast<float*>(t));
+  else k_b0_table<double><<<nb, NCELL, 0, st>>>(grids, blocks, ph, static_cast<double*>(t));
   return cudaGetLastError();
 }
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st) {

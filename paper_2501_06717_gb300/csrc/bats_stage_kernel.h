@@ -259,8 +259,14 @@ __device__ __forceinline__ void b0_at(const PhysDev& ph, const R x[3], R B0[3]) 
     B0[0] = R(q[0]); B0[1] = R(q[1]); B0[2] = R(q[2]);
   } else if (ph.b0 == B0_DIPOLE) {
     R r2 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
-    R r = Ops<R>::sqrt_(r2);
-    R inv_r5 = Ops<R>::div_(R(1), r2 * r2 * r);
+    R inv_r5;
+    if constexpr (std::is_same<R, double>::value) {
+      const double ir = div_sqrt64(1.0, r2), ir2 = ir * ir;
+      inv_r5 = ir2 * ir2 * ir;
+    } else {
+      R r = Ops<R>::sqrt_(r2);
+      inv_r5 = Ops<R>::div_(R(1), r2 * r2 * r);
+    }
     R mr = R(q[0]) * x[0] + R(q[1]) * x[1] + R(q[2]) * x[2];
 #pragma unroll
     for (int c = 0; c < 3; c++) B0[c] = (R(3) * mr * x[c] - R(q[c]) * r2) * inv_r5;
@@ -1043,6 +1049,58 @@ __device__ __forceinline__ void b0_face(const PhysDev& ph, int d, int i, int j, 
   b0_at<R>(ph, x, B0);
 }
 
+// The background field of a cell: B0 at the centre, then div B0 and curl B0 from
+// the face-centre B0 of its six faces (the split-field correction's terms).
+template <class R>
+__device__ __forceinline__ void b0_cell_eval(const PhysDev& ph, const GridDev& G, const BlockDev& B, int c, R o[7]) {
+  const int ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6, lev = B.level;
+  const int gb0 = B.bi * NC, gb1 = B.bj * NC, gb2 = B.bk * NC;
+  R lo0, lo1, lo2, dx0, dx1, dx2, idx0, idx1, idx2;
+  if constexpr (std::is_same<R, double>::value) {
+    lo0 = G.lo[0]; lo1 = G.lo[1]; lo2 = G.lo[2];
+    dx0 = G.dx[lev][0]; dx1 = G.dx[lev][1]; dx2 = G.dx[lev][2];
+    idx0 = G.idx[lev][0]; idx1 = G.idx[lev][1]; idx2 = G.idx[lev][2];
+  } else {
+    lo0 = G.lof[0]; lo1 = G.lof[1]; lo2 = G.lof[2];
+    dx0 = G.dxf[lev][0]; dx1 = G.dxf[lev][1]; dx2 = G.dxf[lev][2];
+    idx0 = G.idxf[lev][0]; idx1 = G.idxf[lev][1]; idx2 = G.idxf[lev][2];
+  }
+  R B0c[3], xm[3], xp[3], ym[3], yp[3], zm[3], zp[3];
+  b0_face<R>(ph, -1, ci, cj, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, B0c);
+  b0_face<R>(ph, 0, ci, cj, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, xm);
+  b0_face<R>(ph, 0, ci + 1, cj, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, xp);
+  b0_face<R>(ph, 1, ci, cj, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, ym);
+  b0_face<R>(ph, 1, ci, cj + 1, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, yp);
+  b0_face<R>(ph, 2, ci, cj, ck, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, zm);
+  b0_face<R>(ph, 2, ci, cj, ck + 1, gb0, gb1, gb2, lo0, lo1, lo2, dx0, dx1, dx2, zp);
+  o[0] = B0c[0];
+  o[1] = B0c[1];
+  o[2] = B0c[2];
+  o[3] = ((xp[0] - xm[0]) * idx0 + (yp[1] - ym[1]) * idx1) + (zp[2] - zm[2]) * idx2;
+  o[4] = (yp[2] - ym[2]) * idx1 - (zp[1] - zm[1]) * idx2;
+  o[5] = (zp[0] - zm[0]) * idx2 - (xp[2] - xm[2]) * idx0;
+  o[6] = (xp[1] - xm[1]) * idx0 - (yp[0] - ym[0]) * idx1;
+}
+static __device__ __noinline__ void b0_cell_eval64(const PhysDev& ph, const GridDev& G, const BlockDev& B, int c,
+                                                   double o[7]) {
+  b0_cell_eval<double>(ph, G, B, c, o);
+}
+// The same from the handle's table: seven coalesced loads instead of seven
+// evaluations of the field (a dipole: two roots and a division each):
+// magnetosphere, 3,872 blocks, mixed 10 steps 6.56 -> 4.97 ms, FP64 2 steps 21.3
+// -> 16.5 ms, for 28 or 56 bytes per cell of reads and of memory.  The FP64
+// form without a table (bats_step_noalloc keeps none) evaluates.
+template <class R>
+__device__ __forceinline__ void b0_cell(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk, int c, R o[7]) {
+  if (std::is_same<R, float>::value || a.b0t) {
+    const R* t = static_cast<const R*>(a.b0t) + static_cast<int64_t>(blk) * (7 * NCELL) + c;
+#pragma unroll
+    for (int k = 0; k < 7; k++) o[k] = t[k * NCELL];
+  } else {
+    if constexpr (std::is_same<R, double>::value) b0_cell_eval64(a.ph, G, B, c, o);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // FP64 form, plain faces.  GB300 runs FP64 at 1/64 of the FP32 rate, so this
 // code is written for the fewest FP64 operations: selections and limiters on
@@ -1818,8 +1876,6 @@ __device__ __forceinline__ float cells_mx_general(const StageArgs& a, const Grid
   double* const dtc = FAST ? nullptr : a.dtc;
   const bool blk_body = FAST ? false : B.body != 0;
   const float idx0 = B.idxf[0], idx1 = B.idxf[1], idx2 = B.idxf[2];
-  const float dxr0 = B.dxf[0], dxr1 = B.dxf[1], dxr2 = B.dxf[2];
-  const float lor0 = G.lof[0], lor1 = G.lof[1], lor2 = G.lof[2];
   const int gb0 = B.bi * NC, gb1 = B.bj * NC, gb2 = B.bk * NC, lev = B.level;
   const float gamma = ph.gammaf;
   // the face values are doubled
@@ -1867,7 +1923,12 @@ __device__ __forceinline__ float cells_mx_general(const StageArgs& a, const Grid
     for (int v = 0; v < NV; v++) Wc[v] = sT[v * NCELL + mx_int(c)];
     float B0c[3] = {0.f, 0.f, 0.f};
     float S[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if constexpr (HAS_B0) b0_face<float>(ph, -1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, B0c);
+    [[maybe_unused]] float b0q[7];
+    if constexpr (HAS_B0) {
+      b0_cell<float>(a, G, B, blk, c, b0q);
+#pragma unroll
+      for (int e = 0; e < 3; e++) B0c[e] = b0q[e];
+    }
     if (ph.powell) {
       float ub1 = Wc[1] * Wc[4] + Wc[2] * Wc[5] + Wc[3] * Wc[6];
 #pragma unroll
@@ -1880,17 +1941,7 @@ __device__ __forceinline__ float cells_mx_general(const StageArgs& a, const Grid
     if constexpr (HAS_B0) {
       // split-field correction from the face-centre B0 of the six faces:
       // S_m += -B1 (div B0)_h + B1 x (curl B0)_h
-      float xm[3], xp[3], ym[3], yp[3], zm[3], zp[3];
-      b0_face<float>(ph, 0, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xm);
-      b0_face<float>(ph, 0, ci + 1, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xp);
-      b0_face<float>(ph, 1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, ym);
-      b0_face<float>(ph, 1, ci, cj + 1, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, yp);
-      b0_face<float>(ph, 2, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zm);
-      b0_face<float>(ph, 2, ci, cj, ck + 1, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zp);
-      float divb0 = ((xp[0] - xm[0]) * idx0 + (yp[1] - ym[1]) * idx1) + (zp[2] - zm[2]) * idx2;
-      float cu0 = (yp[2] - ym[2]) * idx1 - (zp[1] - zm[1]) * idx2;
-      float cu1 = (zp[0] - zm[0]) * idx2 - (xp[2] - xm[2]) * idx0;
-      float cu2 = (xp[1] - xm[1]) * idx0 - (yp[0] - ym[0]) * idx1;
+      const float divb0 = b0q[3], cu0 = b0q[4], cu1 = b0q[5], cu2 = b0q[6];
       float b1x = Wc[4], b1y = Wc[5], b1z = Wc[6];
       S[1] = (S[1] - b1x * divb0) + (b1y * cu2 - b1z * cu1);
       S[2] = (S[2] - b1y * divb0) + (b1z * cu0 - b1x * cu2);
@@ -2731,7 +2782,12 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
           for (int v = 0; v < NV; v++) Wc[v] = sT[v * NTILE + c];
           R B0c[3] = {R(0), R(0), R(0)};
           R S[8] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
-          if constexpr (HAS_B0) b0_face<R>(ph, -1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, B0c);
+          [[maybe_unused]] R b0q[7];
+          if constexpr (HAS_B0) {
+            b0_cell<R>(a, G, B, blk, c, b0q);
+#pragma unroll
+            for (int e = 0; e < 3; e++) B0c[e] = b0q[e];
+          }
           if (ph.powell) {
             R ub1 = Wc[1] * Wc[4] + Wc[2] * Wc[5] + Wc[3] * Wc[6];
 #pragma unroll
@@ -2744,17 +2800,7 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
           if constexpr (HAS_B0) {
             // split-field correction from the face-centre B0 of the six faces:
             // S_m += -B1 (div B0)_h + B1 x (curl B0)_h
-            R xm[3], xp[3], ym[3], yp[3], zm[3], zp[3];
-            b0_face<R>(ph, 0, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xm);
-            b0_face<R>(ph, 0, ci + 1, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, xp);
-            b0_face<R>(ph, 1, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, ym);
-            b0_face<R>(ph, 1, ci, cj + 1, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, yp);
-            b0_face<R>(ph, 2, ci, cj, ck, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zm);
-            b0_face<R>(ph, 2, ci, cj, ck + 1, gb0, gb1, gb2, lor0, lor1, lor2, dxr0, dxr1, dxr2, zp);
-            R divb0 = ((xp[0] - xm[0]) * idx0 + (yp[1] - ym[1]) * idx1) + (zp[2] - zm[2]) * idx2;
-            R cu0 = (yp[2] - ym[2]) * idx1 - (zp[1] - zm[1]) * idx2;
-            R cu1 = (zp[0] - zm[0]) * idx2 - (xp[2] - xm[2]) * idx0;
-            R cu2 = (xp[1] - xm[1]) * idx0 - (yp[0] - ym[0]) * idx1;
+            const R divb0 = b0q[3], cu0 = b0q[4], cu1 = b0q[5], cu2 = b0q[6];
             R b1x = Wc[4], b1y = Wc[5], b1z = Wc[6];
             S[1] = (S[1] - b1x * divb0) + (b1y * cu2 - b1z * cu1);
             S[2] = (S[2] - b1y * divb0) + (b1z * cu0 - b1x * cu2);
