@@ -14,8 +14,9 @@
 //  * k_mlp_train_tc, k_mlp_grad_reduce: the mean-squared-error loss and its
 //    gradient for a batch, every product on tcgen05 (the weight gradients
 //    with the samples as K), per-CTA partial sums added in a fixed order.
-//  * k_mlp_adam, k_mlp_pack: the Adam update of the FP32 master weights and
-//    the BF16 copies in the layouts the kernels read.
+//  * k_mlp_update: a training step's gradient sum, the Adam update of the FP32
+//    master weights and their BF16 copies in the layouts the kernels read
+//    (k_mlp_pack: the copies of given weights).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -263,19 +264,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_mlp_infer(const uint32_t* __r
 }
 
 
-// Adam (Kingma & Ba 2015) on the FP32 master weights, bias-corrected.
-__global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
-                           float* __restrict__ m2, float lr, float b1, float b2, float eps, float c1, float c2) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= MLP_NPARAM) return;
-  float gv = gr[e];
-  float a = b1 * m1[e] + (1.f - b1) * gv;
-  float b = b2 * m2[e] + (1.f - b2) * gv * gv;
-  m1[e] = a;
-  m2[e] = b;
-  p[e] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
-}
-
 // FP32 master weights (W1 [64][40], b1, W2 [64][64], b2, W3 [8][64], b3) ->
 // BF16 pair layouts: w1 [64][24] (inputs 40..47 zero), w2 [64][32],
 // w3 [8][32], w2t [64][32] (transposed), w3t [64][8] (transposed, outputs
@@ -286,6 +274,70 @@ __device__ __forceinline__ uint32_t bias_pair(float b) {
   const float hi = __bfloat162float(__float2bfloat16_rn(b));
   return pack_bf16(hi, b - hi);
 }
+// The BF16 copies (and FP32 biases) of one parameter e of value p, in every layout
+// that holds it (k_mlp_pack's, which also writes the zeros between them).
+__device__ __forceinline__ void put_bf16(uint32_t* w, int word, int half, float v) {
+  reinterpret_cast<__nv_bfloat16*>(w)[2 * word + half] = __float2bfloat16_rn(v);
+}
+__device__ __forceinline__ void pack_param(const MlpDev& m, int e, float p) {
+  constexpr int OB1 = 64 * 40, OW2 = OB1 + 64, OB2 = OW2 + 64 * 64, OW3 = OB2 + 64, OB3 = OW3 + 8 * 64;
+  if (e < OB1) {
+    const int r = e / 40, i = e % 40;
+    put_bf16(m.w1, r * 24 + i / 2, i & 1, p);
+    put_bf16(m.w1b, r * 24 + i / 2, i & 1, p);
+  } else if (e < OW2) {
+    m.b1[e - OB1] = p;
+    m.w1b[(e - OB1) * 24 + 20] = bias_pair(p);
+  } else if (e < OB2) {
+    const int r = (e - OW2) / 64, c = (e - OW2) % 64;
+    put_bf16(m.w2, r * 32 + c / 2, c & 1, p);
+    put_bf16(m.w2t, c * 32 + r / 2, r & 1, p);
+    put_bf16(m.w2b, r * 40 + c / 2, c & 1, 0.5f * p);
+  } else if (e < OW3) {
+    m.b2[e - OB2] = p;
+    m.w2b[(e - OB2) * 40 + 32] = bias_pair(p);
+  } else if (e < OB3) {
+    const int r = (e - OW3) / 64, c = (e - OW3) % 64;
+    put_bf16(m.w3, r * 32 + c / 2, c & 1, p);
+    put_bf16(m.w3t, c * 8 + r / 2, r & 1, p);
+    put_bf16(m.w3b, r * 40 + c / 2, c & 1, 0.5f * p);
+  } else {
+    m.b3[e - OB3] = p;
+    m.w3b[(e - OB3) * 40 + 32] = bias_pair(p);
+  }
+}
+
+// The rest of a training step in one launch, one thread per parameter: its
+// gradient (the partials in CTA order, as k_mlp_grad_reduce), Adam (Kingma & Ba
+// 2015) on the FP32 master weight, bias-corrected, and the BF16 copies.  Three
+// launches (sum, update, copies) made up a third of a step: 14 steps of 8,192
+// samples with four launches each took 709 us, with two 488 us.  CTAs of 64 threads: the sums are chains of loads, spread over the SMs.
+__global__ void __launch_bounds__(64) k_mlp_update(const float* __restrict__ partial,
+                                                   const double* __restrict__ partial_loss, int nparts,
+                                                   double* __restrict__ loss, float* __restrict__ p,
+                                                   float* __restrict__ m1, float* __restrict__ m2, float lr, float b1,
+                                                   float b2, float eps, float c1, float c2, const MlpDev m) {
+  pdl_wait();
+  pdl_next();  // the next step's training pass sets up its shared and tensor memory meanwhile
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < MLP_NPARAM) {
+    float gv = 0.f;
+#pragma unroll 16
+    for (int c = 0; c < nparts; c++) gv += partial[static_cast<int64_t>(c) * MLP_NPARAM + e];
+    const float a = b1 * m1[e] + (1.f - b1) * gv;
+    const float b = b2 * m2[e] + (1.f - b2) * gv * gv;
+    m1[e] = a;
+    m2[e] = b;
+    const float v = p[e] - lr * (a / c1) / (sqrtf(b / c2) + eps);
+    p[e] = v;
+    pack_param(m, e, v);
+  } else if (e == MLP_NPARAM) {
+    double l = 0.0;
+    for (int c = 0; c < nparts; c++) l += partial_loss[c];
+    *loss = l;
+  }
+}
+
 __global__ void k_mlp_pack(const float* __restrict__ P, MlpDev m) {
   const float* W1 = P;
   const float* B1 = W1 + 64 * 40;
@@ -422,8 +474,28 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(const float* __restrict_
   extern __shared__ __align__(128) unsigned char tt_smem_raw[];
   TrainTc& s = *reinterpret_cast<TrainTc*>((reinterpret_cast<uintptr_t>(tt_smem_raw) + 127) & ~uintptr_t(127));
   const int t = threadIdx.x, warp = t >> 5;
-  // weights in the canonical layouts; the constant rows and columns of the
-  // transposed operands (ones, zeros)
+  // the constant rows and columns of the transposed operands (ones, zeros)
+  {
+    const uint16_t one = bf16_bits(1.f);
+    for (int r = 40; r < 48; r++) st_t(s.xt, r, t, r == 40 ? one : 0);
+    for (int r = 64; r < 80; r++) st_t(s.h1t, r, t, r == 64 ? one : 0);
+    for (int r = 64; r < 128; r++) {
+      st_t(s.h2t, r, t, r == 64 ? one : 0);
+      st_t(s.dz2t, r, t, 0);
+      st_t(s.dz1t, r, t, 0);
+    }
+    for (int r = 8; r < 16; r++) st_t(s.dyt, r, t, 0);
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_saddr(&s.tmem)),
+                 "r"(TM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (t == 0) mbar_init_tc(&s.bar);
+  // everything above runs while the update before still does; now the weights, in
+  // the canonical layouts
+  pdl_wait();
   for (int e = t; e < 64 * 6; e += TT) {
     const int r = e / 6, kc = e % 6;
     *reinterpret_cast<uint4*>(s.w1 + cm_off(r, kc, SBO_K48)) = *reinterpret_cast<const uint4*>(m.w1 + r * 24 + kc * 4);
@@ -448,24 +520,6 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(const float* __restrict_
     s.b2[t] = m.b2[t];
   }
   if (t < 8) s.b3[t] = m.b3[t];
-  {
-    const uint16_t one = bf16_bits(1.f);
-    for (int r = 40; r < 48; r++) st_t(s.xt, r, t, r == 40 ? one : 0);
-    for (int r = 64; r < 80; r++) st_t(s.h1t, r, t, r == 64 ? one : 0);
-    for (int r = 64; r < 128; r++) {
-      st_t(s.h2t, r, t, r == 64 ? one : 0);
-      st_t(s.dz2t, r, t, 0);
-      st_t(s.dz1t, r, t, 0);
-    }
-    for (int r = 8; r < 16; r++) st_t(s.dyt, r, t, 0);
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc_saddr(&s.tmem)),
-                 "r"(TM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  if (t == 0) mbar_init_tc(&s.bar);
   proxy_fence_smem();
   tc_fence_before();
   __syncthreads();
@@ -477,6 +531,7 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(const float* __restrict_
   const uint32_t w1s = tc_saddr(s.w1), w2s = tc_saddr(s.w2), w3s = tc_saddr(s.w3), w3ts = tc_saddr(s.w3t),
                  w2ts = tc_saddr(s.w2t);
   const float scale = static_cast<float>(2.0 * inv_count);
+  const bool vec = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
   uint32_t phase = 0;
   bool failed = false, any = false;
   double lsum = 0.0;
@@ -492,8 +547,19 @@ __global__ void __launch_bounds__(TT, 1) k_mlp_train_tc(const float* __restrict_
     // X row t (BF16) as the A of Z1, and its column of [X | 1]^T
     {
       float x[40];
+      if (vec) {  // rows of 160 bytes
 #pragma unroll
-      for (int i = 0; i < 40; i++) x[i] = valid ? X[r * 40 + i] : 0.f;
+        for (int i = 0; i < 10; i++) {
+          const float4 q = valid ? *reinterpret_cast<const float4*>(X + r * 40 + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+          x[4 * i] = q.x;
+          x[4 * i + 1] = q.y;
+          x[4 * i + 2] = q.z;
+          x[4 * i + 3] = q.w;
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 40; i++) x[i] = valid ? X[r * 40 + i] : 0.f;
+      }
 #pragma unroll
       for (int kc = 0; kc < 6; kc++) {
         uint4 o = make_uint4(0u, 0u, 0u, 0u);
@@ -739,25 +805,31 @@ cudaError_t launch_mlp_infer(const uint32_t* X, float* Y, int64_t n, const MlpDe
 // CTA order (the result is the same bit for bit from run to run).  partial:
 // nsm x MLP_NPARAM floats, partial_loss: nsm doubles.
 // idx (nullable, device): sample i is row idx[i] of X and T (nrows rows);
-// without it sample i is row i.
+// without it sample i is row i.  grad == nullptr: the partials only.
 cudaError_t launch_mlp_train(const float* X, const float* T, const int64_t* idx, int64_t nrows, int64_t n,
                              const MlpDev& m, float* grad, double* loss, float* partial, double* partial_loss,
                              int32_t* err, int nsm, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const int64_t tiles = (n + TT - 1) / TT;
   const int grid = static_cast<int>(std::min<int64_t>(tiles, static_cast<int64_t>(nsm)));
-  k_mlp_train_tc<<<grid, TT, kTrainTcSmem, st>>>(X, T, idx, nrows, n, 1.0 / (8.0 * static_cast<double>(n)), m,
-                                                  partial, partial_loss, err);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  cudaError_t e = launch_pdl(k_mlp_train_tc, grid, TT, kTrainTcSmem, st, X, T, idx, nrows, n,
+                             1.0 / (8.0 * static_cast<double>(n)), m, partial, partial_loss, err);
+  if (e != cudaSuccess || !grad) return e;
   k_mlp_grad_reduce<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(partial, partial_loss, grid, grad, loss);
   return cudaGetLastError();
 }
-cudaError_t launch_mlp_adam(float* p, const float* g, float* m1, float* m2, float lr, int step, cudaStream_t st) {
+// One Adam step of the FP32 master weights p on the batch (training pass without
+// a gradient of its own, then the update with the BF16 copies); *loss its loss sum.
+cudaError_t launch_mlp_step(const float* X, const float* T, const int64_t* idx, int64_t nrows, int64_t n,
+                            const MlpDev& m, double* loss, float* partial, double* partial_loss, int32_t* err, int nsm,
+                            float* p, float* m1, float* m2, float lr, int step, cudaStream_t st) {
+  cudaError_t e = launch_mlp_train(X, T, idx, nrows, n, m, nullptr, nullptr, partial, partial_loss, err, nsm, st);
+  if (e != cudaSuccess) return e;
+  const int parts = static_cast<int>(std::min<int64_t>((n + TT - 1) / TT, static_cast<int64_t>(nsm)));
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  float c1 = 1.f - powf(b1, static_cast<float>(step)), c2 = 1.f - powf(b2, static_cast<float>(step));
-  k_mlp_adam<<<(MLP_NPARAM + 255) / 256, 256, 0, st>>>(p, g, m1, m2, lr, b1, b2, eps, c1, c2);
-  return cudaGetLastError();
+  const float c1 = 1.f - powf(b1, static_cast<float>(step)), c2 = 1.f - powf(b2, static_cast<float>(step));
+  return launch_pdl(k_mlp_update, (MLP_NPARAM + 64) / 64, 64, 0, st, static_cast<const float*>(partial),
+                    static_cast<const double*>(partial_loss), parts, loss, p, m1, m2, lr, b1, b2, eps, c1, c2, m);
 }
 
 cudaError_t launch_rows_to_bf16(const float* X, uint32_t* Xb, int64_t n, cudaStream_t st) {
@@ -863,12 +935,17 @@ int copy_in(bats_mlp_t* m, float* dst, const float* src, size_t count) {
   return e == cudaSuccess ? BATS_OK : BATS_ERR_CUDA;
 }
 
-int grad_pass(bats_mlp_t* m, const float* X, const float* T, int64_t n) {
+int batch_in(bats_mlp_t* m, const float* X, const float* T, int64_t n) {
   if (!X || !T || n <= 0) return BATS_ERR_INVALID_ARG;
   int rc = mlp_reserve(m, n);
   if (rc) return rc;
   if ((rc = copy_in(m, m->X, X, static_cast<size_t>(n) * 40)) || (rc = copy_in(m, m->T, T, static_cast<size_t>(n) * 8)))
     return rc;
+  return BATS_OK;
+}
+
+int grad_pass(bats_mlp_t* m, const float* X, const float* T, int64_t n) {
+  if (int rc = batch_in(m, X, T, n)) return rc;
   if (launch_mlp_train(m->X, m->T, nullptr, n, n, m->w, m->G, m->loss, m->partial, m->partial_loss, m->errw,
                        m->nsm, m->stream) != cudaSuccess)
     return BATS_ERR_CUDA;
@@ -1050,11 +1127,11 @@ int bats_mlp_loss_grad(bats_mlp_t* m, const float* X, const float* T, int64_t n,
 
 int bats_mlp_train_step(bats_mlp_t* m, const float* X, const float* T, int64_t n, float lr, double* loss) {
   if (!m || !(lr >= 0.f)) return BATS_ERR_INVALID_ARG;
-  int rc = grad_pass(m, X, T, n);
+  int rc = batch_in(m, X, T, n);
   if (rc) return rc;
   m->step++;
-  if (launch_mlp_adam(m->P, m->G, m->M1, m->M2, lr, m->step, m->stream) != cudaSuccess ||
-      launch_mlp_pack(m->P, m->w, m->stream) != cudaSuccess)
+  if (launch_mlp_step(m->X, m->T, nullptr, n, n, m->w, m->loss, m->partial, m->partial_loss, m->errw, m->nsm, m->P,
+                      m->M1, m->M2, lr, m->step, m->stream) != cudaSuccess)
     return BATS_ERR_CUDA;
   if (loss) {
     double ls = 0.0;
@@ -1083,12 +1160,9 @@ int bats_mlp_train_epoch(bats_mlp_t* m, const float* X, const float* T, int64_t 
     m->step_cap = steps;
   }
   for (int64_t s = 0; s < steps; s++) {
-    if (launch_mlp_train(X, T, perm + s * batch, n, batch, m->w, m->G, m->step_loss + s, m->partial,
-                         m->partial_loss, m->errw, m->nsm, m->stream) != cudaSuccess)
-      return BATS_ERR_CUDA;
     m->step++;
-    if (launch_mlp_adam(m->P, m->G, m->M1, m->M2, lr, m->step, m->stream) != cudaSuccess ||
-        launch_mlp_pack(m->P, m->w, m->stream) != cudaSuccess)
+    if (launch_mlp_step(X, T, perm + s * batch, n, batch, m->w, m->step_loss + s, m->partial, m->partial_loss, m->errw,
+                        m->nsm, m->P, m->M1, m->M2, lr, m->step, m->stream) != cudaSuccess)
       return BATS_ERR_CUDA;
   }
   std::vector<double> ls(static_cast<size_t>(steps));

@@ -584,22 +584,6 @@ static size_t stage_smem(bool mixed, bool lrn) {
   return mixed ? (lrn ? kSmemLx : StageCfg<true>::SMEM_MX) : StageCfg<false>::SMEM;
 }
 
-// Launch of a kernel that begins with pdl_wait or pdl_begin.
-template <class... P, class... A>
-static cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t st, const A&... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3(grid);
-  c.blockDim = dim3(block);
-  c.dynamicSmemBytes = smem;
-  c.stream = st;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  return cudaLaunchKernelEx(&c, k, args...);
-}
-
 using StageFn = void (*)(const StageArgs);
 template <bool MIXED, bool LRN, int FLX>
 StageFn stage_fn_l(int lim, bool b0) {

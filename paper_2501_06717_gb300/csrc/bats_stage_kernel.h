@@ -81,20 +81,6 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// Programmatic dependent launch: the kernels of a step follow one another on one
-// stream and are launched with the attribute that lets the next one start before
-// this one has ended.  pdl_wait, at a kernel's start, waits until the kernels
-// before have completed and their writes are visible; only reads of static
-// tables may stand before it.  (Without the launch attribute it returns at once.)
-// pdl_begin also lets the next kernel start at once: for the short kernels, whose
-// successors then stand ready.  The stage kernels leave that to their end (an
-// early start of what follows them made the 960-block fast wave 13 % slower, the
-// end 3 % faster than ordinary launches).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  pdl_wait();
-}
 // A load that stays where it is written (ahead of a barrier).
 __device__ __forceinline__ double ld_early(const double* p) {
   double v;

@@ -13,6 +13,39 @@
 
 namespace batsk {
 
+// Programmatic dependent launch: the kernels of a step follow one another on one
+// stream and are launched with the attribute that lets the next one start before
+// this one has ended.  pdl_wait, at a kernel's start, waits until the kernels
+// before have completed and their writes are visible; only reads of static
+// tables may stand before it.  (Without the launch attribute it returns at once.)
+// pdl_begin also lets the next kernel start at once: for the short kernels, whose
+// successors then stand ready.  The stage kernels leave that to their end (an
+// early start of what follows them made the 960-block fast wave 13 % slower, the
+// end 3 % faster than ordinary launches).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+  pdl_next();
+  pdl_wait();
+}
+
+// Launch of a kernel that begins with pdl_wait or pdl_begin.
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*k)(P...), int grid, int block, size_t smem, cudaStream_t st, const A&... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, args...);
+}
+
+
 __device__ __forceinline__ uint32_t tc_saddr(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
