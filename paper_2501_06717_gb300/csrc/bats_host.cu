@@ -497,6 +497,20 @@ int launch_stage_one(bats_t* h, const StageArgs& a0, bool make_ghosts = true, bo
     int per_sm = h->ctas_per_sm > 0 ? std::min(h->ctas_per_sm, h->occ[mixed]) : h->occ[mixed];
     grid = std::min(nitems, h->num_sms * std::max(1, per_sm));
   }
+  // FP64 form with at most half as many blocks as SMs: a block is FP64-bound on
+  // its one SM, so 2, 4 or 8 CTAs share it, by layers of cells, as long as all of
+  // them run at once (one step of 8 blocks with its state in and out: 304 us
+  // whole, 149 us in eight parts).  A layer split computes the faces between two
+  // parts twice and every slope for both of its faces; 120 blocks in four parts
+  // on 152 SMs would take four rounds of more than a quarter.
+  if (!mixed && !a.learned && a.kind < 3) {
+    a.parts = 8;
+    while (a.parts > 1 && a.nblocks * a.parts > h->num_sms) a.parts /= 2;
+    if (a.parts > 1) {
+      a.blocks_per_item = 1;
+      grid = a.nblocks * a.parts;
+    }
+  }
   if (grid <= 0) return BATS_OK;
   h->launches++;
   CK(h, launch_stage_kernel(mixed, grid, h->stream, a));

@@ -124,6 +124,7 @@ struct StageArgs {
   int32_t* err;           // [0] error bits, [1] first bad block
   int32_t nblocks;
   int32_t blocks_per_item;
+  int32_t parts;          // plain FP64 stage: CTAs per block (2, 4 or 8: 4, 2 or 1 layers of cells each), else 0 or 1
   int32_t kind;           // 0: Uout = Ubase + c R;  1: Uout = 0.5 Ubase + 0.5 (Uin + c R);
                           // 2: Uout = R (debug);  3: face features only (Xb);
                           // 4: features and plain fluxes only (Xf, Fd)

@@ -188,13 +188,13 @@ __device__ __forceinline__ double div_sqrt64(double a, double x) {
   const double r = fma(-(x * y), y, 1.0);
   return fma(fma(0.375, r, 0.5), r * c, c);
 }
-// Fast magnetosonic speed from half the sound term (gamma/2) p, half of B^2,
-// the squared normal field and rho:
+// Fast magnetosonic speed from half the sound term (gamma/2) p, B^2, the squared
+// normal field and rho:
 //   c_f^2 = (G + sqrt(G^2 - gamma p B_n^2)) / rho,  G = (gamma p + B^2) / 2,
 // the usual form with 1/rho taken out of both roots, which leaves no division
 // (c_f = Q / sqrt(Q rho)).
-__device__ __forceinline__ double fast_speed64(double gph, double hbsq, double bn2, double rho) {
-  const double G = gph + hbsq;
+__device__ __forceinline__ double fast_speed64(double gph, double bsq, double bn2, double rho) {
+  const double G = fma(0.5, bsq, gph);
   double D = fma(-2.0, gph * bn2, G * G);
   D = __double2hiint(D) < 0 ? 0.0 : D;
   const double Q = G + sqrt64(D);
@@ -346,10 +346,10 @@ __device__ __forceinline__ float fast_speed_n(float gamma, float rho, float p, f
 // CFL bound of a cell, sum_d (|u_d| + c_f,d) / dx_d, with the total field B.
 __device__ __forceinline__ double cfl_sum64(double gamma, const double W[8], const double B[3], const double idx[3]) {
   const double b2[3] = {B[0] * B[0], B[1] * B[1], B[2] * B[2]};
-  const double gph = 0.5 * gamma * W[7], hb = 0.5 * (b2[0] + b2[1] + b2[2]);
+  const double gph = 0.5 * gamma * W[7], bsq = b2[0] + b2[1] + b2[2];
   double s = 0.0;
 #pragma unroll
-  for (int d = 0; d < 3; d++) s = fma(fabs(W[1 + d]) + fast_speed64(gph, hb, b2[d], W[0]), idx[d], s);
+  for (int d = 0; d < 3; d++) s = fma(fabs(W[1 + d]) + fast_speed64(gph, bsq, b2[d], W[0]), idx[d], s);
   return s;
 }
 
@@ -402,6 +402,14 @@ __device__ __forceinline__ double minmod_d(double a, double b) {
   long long r = ma < mb ? ia : ib;
   return same ? __longlong_as_double(r) : 0.0;
 }
+// Comparisons of doubles on bit patterns (a comparison shares the FP64 pipe,
+// which bounds the FP64 form): the order of non-NaN values as signed integers.
+__device__ __forceinline__ long long order_d(double x) {
+  const long long i = __double_as_longlong(x);
+  return i ^ ((i >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double max_d(double a, double b) { return order_d(a) > order_d(b) ? a : b; }
+__device__ __forceinline__ double min_d(double a, double b) { return order_d(a) < order_d(b) ? a : b; }
 // Validity tests on bit patterns: finite, and finite and > 0.
 __device__ __forceinline__ bool finite_d(double x) {
   return (static_cast<unsigned>(__double2hiint(x)) & 0x7ff00000u) != 0x7ff00000u;
@@ -1134,8 +1142,7 @@ __device__ __forceinline__ void side64(const double w[8], const double B0[3], do
     tt0 = T0 * T0;
     tsq = fma(T2, T2, fma(T1, T1, tt0));
   }
-  cf = fast_speed64(hgamma * p, 0.5 * tsq, tt0, rho);
-  const double usq = fma(u2, u2, fma(u1, u1, u0 * u0));
+  cf = fast_speed64(hgamma * p, tsq, tt0, rho);
   const double ub = fma(u2, b2, fma(u1, b1, u0 * b0));
   double pt = fma(0.5, bsq, p);
   if constexpr (HAS_B0) pt = fma(B0[2], b2, fma(B0[1], b1, fma(B0[0], b0, pt)));
@@ -1146,7 +1153,7 @@ __device__ __forceinline__ void side64(const double w[8], const double B0[3], do
   U[4] = b0;
   U[5] = b1;
   U[6] = b2;
-  U[7] = fma(p, inv_gm1, 0.5 * fma(rho, usq, bsq));
+  U[7] = fma(p, inv_gm1, 0.5 * fma(U[3], u2, fma(U[2], u1, fma(U[1], u0, bsq))));
   F[0] = U[1];
   F[1] = fma(U[1], u0, fma(-b0, T0, pt));
   F[2] = fma(U[2], u0, -(b1 * T0));
@@ -1162,8 +1169,10 @@ __device__ __forceinline__ void side64(const double w[8], const double B0[3], do
   F[7] = fma(u0, U[7] + pt, -(ub * T0));
 }
 
-// Twice the numerical flux of the face with left and right states wl, wr;
-// Rusanov: also cmax and dU = U_R - U_L (for the learned correction's clip).
+// fscale64 times the numerical flux of the face with left and right states wl, wr
+// (Rusanov: twice, which saves its halving; the cell phase halves its spacing
+// instead); Rusanov: also cmax and dU = U_R - U_L (for the learned correction's clip).
+constexpr double fscale64(int flx) { return flx == FLUX_RUSANOV ? 2.0 : 1.0; }
 template <bool HAS_B0, int FLX>
 __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[8], const double B0[3], double hgamma,
                                             double inv_gm1, double G[8], double& cmax, double dU[8]) {
@@ -1173,17 +1182,13 @@ __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[
   if constexpr (FLX == FLUX_HLL || FLX == FLUX_LINDE) {
     // HLL with S_L = min(unL - cfL, unR - cfR, 0), S_R = max(unL + cfL, unR +
     // cfR, 0):  F = F_L - S_L/(S_R - S_L) ((F_R - F_L) - S_R (U_R - U_L))
-    double sl = wl[1] - cl < wr[1] - cr ? wl[1] - cl : wr[1] - cr;
-    double sr = wl[1] + cl > wr[1] + cr ? wl[1] + cl : wr[1] + cr;
-    sl = sl < 0.0 ? sl : 0.0;
-    sr = sr > 0.0 ? sr : 0.0;
+    const double sl = min_d(min_d(wl[1] - cl, wr[1] - cr), 0.0), sr = max_d(max_d(wl[1] + cl, wr[1] + cr), 0.0);
     const double den = sr - sl;
-    const double rden = den > 0.0 ? rcp64(den) : 0.0;
-    const double k2 = 2.0 * (sl * rden);
+    const double kk = __double_as_longlong(den) > 0 ? sl * rcp64(den) : 0.0;
 #pragma unroll
     for (int v = 0; v < NV; v++) {
-      const double dF = v == 4 ? 0.0 : FR[v] - FL[v];
-      G[v] = fma(-k2, fma(-sr, UR[v] - UL[v], dF), v == 4 ? 0.0 : 2.0 * FL[v]);
+      const double dU = UR[v] - UL[v];
+      G[v] = v == 4 ? kk * (sr * dU) : fma(-kk, fma(-sr, dU, FR[v] - FL[v]), FL[v]);
     }
     if constexpr (FLX == FLUX_LINDE) {
       // Linde: the contact wave restored, F -= delta alpha S_L S_R / (S_R - S_L) r,
@@ -1195,7 +1200,7 @@ __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[
       const double cs = div_sqrt64(gp, gp * rm), ic2 = rm * rcp64(gp);
       const double dr = wr[0] - wl[0];
       const double alpha = minmod_d(fma(-(wr[7] - wl[7]), ic2, dr), dr);
-      const double q = k2 == 0.0 ? 0.0 : k2 * sr * alpha * (cs * rcp64(cs + fabs(um0)));
+      const double q = kk == 0.0 ? 0.0 : kk * sr * alpha * (cs * rcp64(cs + fabs(um0)));
       G[0] -= q;
       G[1] = fma(-q, um0, G[1]);
       G[2] = fma(-q, um1, G[2]);
@@ -1204,11 +1209,47 @@ __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[
     }
   } else {
     const double al = fabs(wl[1]) + cl, ar = fabs(wr[1]) + cr;
-    cmax = al > ar ? al : ar;
+    cmax = max_d(al, ar);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       dU[v] = UR[v] - UL[v];
       G[v] = v == 4 ? -cmax * dU[v] : fma(-cmax, dU[v], FL[v] + FR[v]);
+    }
+  }
+}
+
+// Face f of the line (ta, tb) of direction d from its two states: flux and (with
+// the Powell terms) normal B1 into the face arrays, the block-face flux of a
+// resolution change into the flux register.
+template <bool HAS_B0, int FLX>
+__device__ __forceinline__ void put_face64(const StageArgs& a, const BlockDev& B, const double WL[8],
+                                           const double WR[8], double* sF, int d, int ta, int tb, int f,
+                                           double hgamma, double inv_gm1, const double lo[3], const double dx[3]) {
+  const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+  const int rot[8] = {0, 1 + d, 1 + d1, 1 + d2, 4 + d, 4 + d1, 4 + d2, 7};
+  double B0r[3] = {0.0, 0.0, 0.0};
+  if constexpr (HAS_B0) {
+    const int ci = d == 0 ? f : ta, cj = d == 1 ? f : (d == 0 ? ta : tb), ck = d == 2 ? f : tb;
+    double B0f[3];
+    b0_face<double>(a.ph, d, ci, cj, ck, B.bi * NC, B.bj * NC, B.bk * NC, lo[0], lo[1], lo[2], dx[0], dx[1], dx[2],
+                    B0f);
+    B0r[0] = d == 0 ? B0f[0] : (d == 1 ? B0f[1] : B0f[2]);
+    B0r[1] = d1 == 0 ? B0f[0] : (d1 == 1 ? B0f[1] : B0f[2]);
+    B0r[2] = d2 == 0 ? B0f[0] : (d2 == 1 ? B0f[1] : B0f[2]);
+  }
+  double G[8], cmax, dU[8];
+  face_flux64<HAS_B0, FLX>(WL, WR, B0r, hgamma, inv_gm1, G, cmax, dU);
+  double* o = sF + d * (9 * NFACE) + chki((tb * NC + ta) * 9 + f, 0, NFACE);
+#pragma unroll
+  for (int v = 0; v < NV; v++) o[rot[v] * NFACE] = G[v];
+  if (a.ph.powell) o[8 * NFACE] = fscale64(FLX) == 2.0 ? WL[4] + WR[4] : 0.5 * (WL[4] + WR[4]);  // its normal B1
+  // refluxing: the block-face fluxes of faces at resolution changes
+  if (a.freg && (f == 0 || f == NC)) {
+    const int sl = chki(B.rslot[2 * d + (f == NC ? 1 : 0)], -1, a.nslots);
+    if (sl >= 0) {
+      double* r = a.freg + (static_cast<int64_t>(sl) * 64 + ta * NC + tb) * NV;
+#pragma unroll
+      for (int v = 0; v < NV; v++) r[rot[v]] = (1.0 / fscale64(FLX)) * G[v];
     }
   }
 }
@@ -1267,37 +1308,67 @@ __device__ __forceinline__ void faces64(const StageArgs& a, const BlockDev& B, c
         df[v] = dn;
       }
     }
-    double B0r[3] = {0.0, 0.0, 0.0};
-    if constexpr (HAS_B0) {
-      const int ci = d == 0 ? f : ta, cj = d == 1 ? f : (d == 0 ? ta : tb), ck = d == 2 ? f : tb;
-      double B0f[3];
-      b0_face<double>(a.ph, d, ci, cj, ck, B.bi * NC, B.bj * NC, B.bk * NC, lo[0], lo[1], lo[2], dx[0], dx[1], dx[2],
-                      B0f);
-      B0r[0] = d == 0 ? B0f[0] : (d == 1 ? B0f[1] : B0f[2]);
-      B0r[1] = d1 == 0 ? B0f[0] : (d1 == 1 ? B0f[1] : B0f[2]);
-      B0r[2] = d2 == 0 ? B0f[0] : (d2 == 1 ? B0f[1] : B0f[2]);
-    }
-    double G[8], cmax, dU[8];
-    face_flux64<HAS_B0, FLX>(WL, WR, B0r, hgamma, inv_gm1, G, cmax, dU);
-    double* o = sF + d * (9 * NFACE) + chki(fline * 9 + f, 0, NFACE);
-#pragma unroll
-    for (int v = 0; v < NV; v++) o[rot[v] * NFACE] = G[v];
-    if (a.ph.powell) o[8 * NFACE] = WL[4] + WR[4];  // twice the face's normal B1
-    // refluxing: the block-face fluxes of faces at resolution changes
-    if (a.freg && (f == 0 || f == NC)) {
-      const int sl = chki(B.rslot[2 * d + (f == NC ? 1 : 0)], -1, a.nslots);
-      if (sl >= 0) {
-        double* r = a.freg + (static_cast<int64_t>(sl) * 64 + ta * NC + tb) * NV;
-#pragma unroll
-        for (int v = 0; v < NV; v++) r[rot[v]] = 0.5 * G[v];
-      }
-    }
+    put_face64<HAS_B0, FLX>(a, B, WL, WR, sF, d, ta, tb, f, hgamma, inv_gm1, lo, dx);
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       WL[v] = WLn[v];
       W0[v] = Wp[v];
     }
   }
+}
+
+// The faces that the cells of layers k0 .. k0 + nk - 1 of a split block need, one
+// face per thread and turn (few blocks: the work of one block over several SMs,
+// and on each over all threads at once, at the price of every slope computed
+// for both of its faces): whole warps of x, then y, then z faces.
+template <int LIM, bool HAS_B0, int FLX>
+__device__ __forceinline__ void faces64_layers(const StageArgs& a, const BlockDev& B, const double* sT, double* sF,
+                                               int k0, int nk, int tid, double hgamma, double inv_gm1,
+                                               const double lo[3], const double dx[3]) {
+  const int wxy = (72 * nk + 31) / 32, warps = 2 * wxy + 2 * (nk + 1);
+  for (int w = tid >> 5; w < warps; w += FACE_THREADS / 32) {
+    const int d = w < wxy ? 0 : (w < 2 * wxy ? 1 : 2);
+    const int e = 32 * (w - d * wxy) + (tid & 31);
+    int ta, tb, f;
+    if (d < 2) {
+      if (e >= 72 * nk) continue;
+      const int line = e / 9;
+      f = e - 9 * line;
+      ta = line & 7;
+      tb = k0 + (line >> 3);
+    } else {
+      ta = e & 7;
+      tb = (e >> 3) & 7;
+      f = k0 + (e >> 6);
+    }
+    const int d1 = d == 2 ? 0 : d + 1, d2 = d == 0 ? 2 : d - 1;
+    const int rot[8] = {0, 1 + d, 1 + d1, 1 + d2, 4 + d, 4 + d1, 4 + d2, 7};
+    const int i0 = chki(tile_index(d, f - 2, ta, tb), 0, NTILE), i1 = chki(tile_index(d, f - 1, ta, tb), 0, NTILE),
+              i2 = chki(tile_index(d, f, ta, tb), 0, NTILE), i3 = chki(tile_index(d, f + 1, ta, tb), 0, NTILE);
+    double WL[8], WR[8];
+#pragma unroll
+    for (int v = 0; v < NV; v++) {
+      const double* q = sT + rot[v] * NTILE;
+      const double w1 = q[i1], w2 = q[i2];
+      if constexpr (LIM == 2) {
+        WL[v] = w1;
+        WR[v] = w2;
+      } else {
+        double f1, f2;
+        const double df = w2 - w1;
+        const double h1 = half_slope64<LIM>(w1 - q[i0], df, f1), h2 = half_slope64<LIM>(df, q[i3] - w2, f2);
+        WL[v] = fma(f1, h1, w1);
+        WR[v] = fma(-f2, h2, w2);
+      }
+    }
+    put_face64<HAS_B0, FLX>(a, B, WL, WR, sF, d, ta, tb, f, hgamma, inv_gm1, lo, dx);
+  }
+}
+// Whether layers k0 .. k0 + nk - 1 read tile cell c (interior or face slab).
+__device__ __forceinline__ bool layers_need(int c, int k0, int nk) {
+  if (c < NCELL) return (c >> 6) >= k0 - 2 && (c >> 6) < k0 + nk + 2;
+  const int q = c - NCELL, s = q >> 7, tb = (q & 127) >> 4;
+  return s < 4 ? tb >= k0 && tb < k0 + nk : (s == 4 ? k0 < 2 : k0 + nk > NC - 2);
 }
 
 // ---------------------------------------------------------------------------
@@ -2425,10 +2496,14 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
   }
   uint32_t parity = 0;
 
-  const int nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
+  // plain FP64 form: parts > 1 CTAs share a block, this one its layers k0 .. k0 + nk - 1
+  const int parts = !MIXED && !LRN && a.parts > 1 ? a.parts : 1;
+  const int nk = NC / parts;
+  const int nitems = (a.nblocks * parts + a.blocks_per_item - 1) / a.blocks_per_item;
   for (int item = blockIdx.x; item < nitems; item += gridDim.x) {
-    const int b_end = min(a.nblocks, (item + 1) * a.blocks_per_item);
-    for (int blk = item * a.blocks_per_item; blk < b_end; blk++) {
+    const int b_end = min(a.nblocks * parts, (item + 1) * a.blocks_per_item);
+    for (int bp = item * a.blocks_per_item; bp < b_end; bp++) {
+      const int blk = bp / parts, k0 = (bp - blk * parts) * nk;
       const BlockDev& B = a.blocks[blk];
       const GridDev& G = a.grids[B.grid];
       GhostCtx cx{&G, a.blocks, a.levmap, a.Uin, a.err};
@@ -2463,8 +2538,8 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
       if (tid == 0) {
         // this CTA's next block: its interior on its way to L2 while this
         // block is computed, so that its bulk copies read L2, not HBM
-        const int nblk = blk + 1 < b_end ? blk + 1 : (item + static_cast<int>(gridDim.x)) * a.blocks_per_item;
-        if (nblk < a.nblocks) {
+        const int nblk = bp + 1 < b_end ? bp + 1 : (item + static_cast<int>(gridDim.x)) * a.blocks_per_item;
+        if (parts == 1 && nblk < a.nblocks) {
           const R* nsrc = MIXED ? reinterpret_cast<const R*>(a.Win) : reinterpret_cast<const R*>(a.Uin);
           prefetch_l2(nsrc + static_cast<int64_t>(nblk) * (NV * NCELL), NV * NCELL * sizeof(R));
         }
@@ -2483,6 +2558,7 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
       // 2. FP64 form: primitives in place over the whole tile
       if constexpr (!MIXED) {
         for (int c = tid; c < NTILE; c += STAGE_THREADS) {
+          if (!layers_need(c, k0, nk)) continue;
           double U[8], W[8];
 #pragma unroll
           for (int v = 0; v < NV; v++) U[v] = sT[v * NTILE + c];
@@ -2720,8 +2796,8 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
         const int kind = FAST ? 0 : a.kind;
         double* const dtc = FAST ? nullptr : a.dtc;
         const bool blk_body = FAST ? false : B.body != 0;
-        // the plain face phases store doubled face values
-        constexpr R FS = LRN ? R(1) : R(0.5);
+        // the plain face phase stores scaled face values
+        constexpr R FS = LRN ? R(1) : R(1.0 / fscale64(FLX));
         const R fidx0 = FS * idx0, fidx1 = FS * idx1, fidx2 = FS * idx2;
         bool any_bad = false;
         R smax_loc = R(0);
@@ -2731,7 +2807,7 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
         // (the FP64 state is read and accumulated in the last stage only)
         [[maybe_unused]] const bool light = MIXED && kind == 0 && !a.last && !a.write_u_all;
         const float c32_blk = d2f_int(cdt_blk);
-        for (int c = tid; c < NCELL; c += STAGE_THREADS) {
+        for (int c = NC * NC * k0 + tid; c < NC * NC * (k0 + nk); c += STAGE_THREADS) {
           // local time stepping: this cell's own dt
           const double cdt = dtc ? a.beta * dtc[static_cast<int64_t>(blk) * NCELL + c] : cdt_blk;
           const float c32 = dtc ? d2f_int(cdt) : c32_blk;
@@ -2927,7 +3003,10 @@ __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constan
         if (tid < FACE_THREADS) {
           const double lo[3] = {lor0, lor1, lor2}, dx[3] = {dxr0, dxr1, dxr2};
           const int wq = (tid >> 5) & 3;
-          faces64<LIM, HAS_B0, FLX>(a, B, sT, sF, fd, 32 * (wq & 1) + (tid & 31), (wq >> 1) ^ (fd & 1), 0.5 * gamma,
+          if (parts > 1)
+            faces64_layers<LIM, HAS_B0, FLX>(a, B, sT, sF, k0, nk, tid, 0.5 * gamma, inv_gm1, lo, dx);
+          else
+            faces64<LIM, HAS_B0, FLX>(a, B, sT, sF, fd, 32 * (wq & 1) + (tid & 31), (wq >> 1) ^ (fd & 1), 0.5 * gamma,
                                     inv_gm1, lo, dx);
         }
       } else {
