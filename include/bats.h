@@ -96,6 +96,11 @@ typedef struct {
  *  persistent     1 = one persistent launch per stage (grid = SMs x occupancy)
  *  blocks_per_cta blocks processed per work item in the persistent launch (>= 1)
  *  ctas_per_sm    persistent CTAs per SM (0 = the occupancy limit)
+ *                 (These three change neither results nor what is accepted.  The
+ *                 mixed form's plain stage always walks the work items with one
+ *                 CTA per SM, of at most as many blocks as leave a CTA eight
+ *                 items; a plain FP64 handle of at most half as many blocks as the
+ *                 GPU has SMs shares each block among 2, 4 or 8 CTAs.)
  *  use_graph      1 = replay whole bats_step calls from a CUDA graph
  *  local_dt       1 = local time stepping (Section 5.2's steady-state session):
  *                 with a CFL number, every cell advances with its own

@@ -7,6 +7,8 @@ inside the library bracket the stage kernels) and keeps the fastest:
   blocks_per_cta blocks per work item (consecutive blocks in leaf order, which
                  is a space-filling order, so neighbours' halos hit in L2)
   ctas_per_sm    persistent CTAs per SM (0 = the occupancy limit)
+                 (the mixed form's plain stage always walks its work items with
+                 one CTA per SM: there the first two differ little)
   staging        mixed form only: how the stage kernel stages each block's
                  padded stencil in shared memory -- 1 = the same-level face
                  slabs by tensor copies (TMA), 0 = gathered by the threads
