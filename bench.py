@@ -602,7 +602,7 @@ def main():
                        "cfl": cfl},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel": ("k_stage<true> with its ghost pre-pass k_amr_ghosts" if prec == bats.BATS_MIXED
+                         "kernel": ("k_stage_mx with its ghost pre-pass k_amr_ghosts" if prec == bats.BATS_MIXED
                                     else "k_stage<false>"),
                          "peak_source": peak_kind, "bytes_per_launch": alg_bytes,
                          "mean_launch_ms": per_launch_ms},
