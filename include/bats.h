@@ -233,6 +233,12 @@ int bats_debug_residual(bats_t* h, int grid, double* R, size_t n);
  * BATS_ERR_TIMEOUT after about 1 s; the handle stays usable. */
 int bats_debug_wait_timeout(bats_t* h);
 
+/* Test hook for the mixed stage's warp-wide wait: a warp waits (about 1 s at
+ * most) on a barrier that another warp of its CTA completes after delay_s
+ * seconds (0..3); lanes[i] is lane i's answer (1 completed, 0 gave up), the same
+ * in all lanes.  Returns BATS_ERR_TIMEOUT if the wait ran out. */
+int bats_debug_wait_warp(bats_t* h, double delay_s, int32_t lanes[32]);
+
 /* Launch-form controls (the autotuner's knobs): persistent launch on/off,
  * blocks per work item, CTAs per SM, CUDA-graph replay of whole steps. */
 int bats_set_launch(bats_t* h, int persistent, int blocks_per_cta, int ctas_per_sm, int use_graph);

@@ -106,6 +106,7 @@ def lib():
     L.bats_debug_fill_ghosts_w.argtypes = [vp, ctypes.c_int, dp, ctypes.c_size_t]
     L.bats_debug_residual.argtypes = [vp, ctypes.c_int, dp, ctypes.c_size_t]
     L.bats_debug_wait_timeout.argtypes = [vp]
+    L.bats_debug_wait_warp.argtypes = [vp, ctypes.c_double, vp]
     L.bats_set_launch.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int]
     L.bats_set_staging.argtypes = [vp, ctypes.c_int]
     L.bats_fp64_fma_rate.argtypes = [vp, ctypes.POINTER(ctypes.c_double)]
@@ -292,6 +293,14 @@ def bats_debug_fill_ghosts_w(h, grid, out):
 
 def bats_debug_wait_timeout(h):
     _check(h, lib().bats_debug_wait_timeout(h))
+
+
+def bats_debug_wait_warp(h, delay_s):
+    """(status code, the 32 lanes' answers) of a warp's wait on a barrier that
+    completes after delay_s seconds."""
+    lanes = np.zeros(32, dtype=np.int32)
+    rc = lib().bats_debug_wait_warp(h, float(delay_s), lanes.ctypes.data)
+    return rc, lanes
 
 
 def bats_debug_residual(h, grid, out):

@@ -49,6 +49,7 @@ cudaError_t launch_check_conversions(const float* f, const double* d, int n, dou
 cudaError_t launch_fp64_fma_rate(double* out, int ctas, int iters, cudaStream_t st);
 cudaError_t read_index_flag(int32_t* out);
 cudaError_t launch_debug_wait_timeout(int32_t* err, cudaStream_t st);
+cudaError_t launch_debug_wait_warp(int32_t* err, int32_t* lanes, unsigned long long delay_ns, cudaStream_t st);
 cudaError_t mlp_alloc(MlpDev* w);
 cudaError_t mlp_setup();
 void mlp_free(MlpDev* w);
@@ -1167,6 +1168,21 @@ int bats_debug_wait_timeout(bats_t* h) {
   CK(h, launch_debug_wait_timeout(h->errw, h->stream));
   int32_t ew[3];
   CK(h, cudaMemcpyAsync(ew, h->errw, sizeof(ew), cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaStreamSynchronize(h->stream));
+  if (ew[0] & ERR_TIMEOUT) return fail(h, BATS_ERR_TIMEOUT, "a bounded device wait ran out");
+  return BATS_OK;
+}
+
+int bats_debug_wait_warp(bats_t* h, double delay_s, int32_t lanes[32]) {
+  if (!h) return BATS_ERR_INVALID_ARG;
+  if (!lanes || !(delay_s >= 0.0 && delay_s <= 3.0)) return fail(h, BATS_ERR_INVALID_ARG, "delay out of 0..3 s");
+  int32_t* d = reinterpret_cast<int32_t*>(h->staging);  // (holds at least one block's tile)
+  int32_t init[3] = {0, INT_MAX, 0};
+  CK(h, cudaMemcpyAsync(h->errw, init, sizeof(init), cudaMemcpyHostToDevice, h->stream));
+  CK(h, launch_debug_wait_warp(h->errw, d, static_cast<unsigned long long>(delay_s * 1e9), h->stream));
+  int32_t ew[3];
+  CK(h, cudaMemcpyAsync(ew, h->errw, sizeof(ew), cudaMemcpyDeviceToHost, h->stream));
+  CK(h, cudaMemcpyAsync(lanes, d, 32 * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   if (ew[0] & ERR_TIMEOUT) return fail(h, BATS_ERR_TIMEOUT, "a bounded device wait ran out");
   return BATS_OK;

@@ -742,6 +742,24 @@ cudaError_t launch_debug_wait_timeout(int32_t* err, cudaStream_t st) {
   k_debug_wait_timeout<<<1, 32, 0, st>>>(err);
   return cudaGetLastError();
 }
+// Hook for the warp-wide wait: lanes[i] = whether lane i was told that the barrier
+// completed; a second warp arrives delay_ns after the start.
+__global__ void __launch_bounds__(64) k_debug_wait_warp(int32_t* err, int32_t* lanes, unsigned long long delay_ns) {
+  __shared__ uint64_t bar;
+  if (threadIdx.x == 0) mbar_init(&bar, 1);
+  __syncthreads();
+  if (threadIdx.x >= 32) {
+    const uint64_t t0 = globaltimer();
+    while (globaltimer() - t0 < delay_ns) __nanosleep(200);
+    if (threadIdx.x == 32) mbar_arrive(&bar);
+  } else {
+    lanes[threadIdx.x] = mbar_wait_warp<false>(&bar, 0, err);
+  }
+}
+cudaError_t launch_debug_wait_warp(int32_t* err, int32_t* lanes, unsigned long long delay_ns, cudaStream_t st) {
+  k_debug_wait_warp<<<1, 64, 0, st>>>(err, lanes, delay_ns);
+  return cudaGetLastError();
+}
 
 // FP64 FMA throughput probe (the FP64 form's roofline): every thread runs
 // `iters` rounds of eight independent FMA chains x = x * b + c, so that the

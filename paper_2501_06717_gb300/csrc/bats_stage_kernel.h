@@ -115,6 +115,29 @@ __device__ __forceinline__ bool mbar_wait_inline(uint64_t* bar, uint32_t parity,
 static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, int32_t* err) {
   return mbar_wait_inline(bar, parity, err);
 }
+// The wait of a whole converged warp, with one answer for all lanes: the code
+// after it branches on the answer around warp collectives.  Done when every lane
+// has seen the phase; lane 0's clock decides when to give up.  LOOP_INLINE: the
+// polls after the first are inline (64 grids, no B0: 1.6 % slower than a call;
+// magnetosphere, dipole B0: 1.6 % faster).
+__device__ __forceinline__ bool mbar_poll_warp(uint64_t* bar, uint32_t parity, int32_t* err) {
+  const uint64_t t0 = globaltimer();
+  while (true) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__shfl_sync(0xffffffffu, globaltimer() - t0 > 1000000000ull, 0)) {
+      if ((threadIdx.x & 31) == 0) atomicOr(err, ERR_TIMEOUT);
+      return false;
+    }
+  }
+}
+static __device__ __noinline__ bool mbar_poll_warp_call(uint64_t* bar, uint32_t parity, int32_t* err) {
+  return mbar_poll_warp(bar, parity, err);
+}
+template <bool LOOP_INLINE>
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int32_t* err) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  return LOOP_INLINE ? mbar_poll_warp(bar, parity, err) : mbar_poll_warp_call(bar, parity, err);
+}
 
 // ---------------------------------------------------------------------------
 // Conversions without the FP64 pipe.  On GB300 the F2F instructions share the
@@ -2100,8 +2123,9 @@ __device__ __forceinline__ float cells_mx_general(const StageArgs& a, const Grid
 // handed over through mbarriers: full (copies landed; faces done by the 12
 // warps) and empty (tile read by the 12 face warps and the 8 parts; face values
 // read by the 8 parts).  Shared memory (2 x (48 + 61) KB) bounds the depth.
-// Every wait is bounded: a warp whose wait ran out flags it, skips its work and
-// further waits from then on, but keeps arriving, so that every warp ends.
+// Every wait is bounded and has one answer per warp: a warp whose wait ran out
+// flags it, skips its work and further waits from then on, but keeps arriving, so
+// that every warp ends.
 constexpr int MX_PARTS = 8;
 struct MxBars {
   uint64_t tile_full[2], tile_empty[2], face_full[2], face_empty[2], slabs[2];
@@ -2130,15 +2154,16 @@ __global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constan
   __syncthreads();
   pdl_wait();
   const int nitems = (a.nblocks + a.blocks_per_item - 1) / a.blocks_per_item;
-  bool failed = false;
+  bool failed = false;  // the same in all lanes of a warp
   auto wait = [&](uint64_t* b, uint32_t parity) {
-    if (!failed) failed = !mbar_wait_inline(b, parity, a.err);
+    if (!failed) failed = !mbar_wait_warp<HAS_B0>(b, parity, a.err);
   };
   // two barriers, the first polls in flight together
   auto wait2 = [&](uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, bool second) {
     const bool r0 = mbar_try_wait(b0, p0), r1 = !second || mbar_try_wait(b1, p1);
-    if (!failed && !r0) failed = !mbar_wait_inline(b0, p0, a.err);
-    if (!failed && !r1) failed = !mbar_wait_inline(b1, p1, a.err);
+    if (__all_sync(0xffffffffu, r0 && r1)) return;
+    wait(b0, p0);
+    if (second) wait(b1, p1);
   };
   // the CTA's n blocks: items of bpi consecutive blocks, every gridDim.x-th one
   const int bpi = a.blocks_per_item;
@@ -2149,13 +2174,14 @@ __global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constan
     const int it = q / bpi;
     return (static_cast<int>(blockIdx.x) + it * static_cast<int>(gridDim.x)) * bpi + (q - it * bpi);
   };
-  // one thread: the copies of the CTA's q-th block, once its tile is free
+  // one thread (lane 0, whose `failed` the warp then takes over): the copies of
+  // the CTA's q-th block, once its tile is free
   const bool reads_ubase = !(a.kind == 0 && !a.last && !a.write_u_all);
   auto issue = [&](int q) {
     const int b = q & 1, blk = block_of(q);
     const MxPlan plan = mx_plan(a, blk);
     const unsigned fill = mx_fill_mask(a, plan);
-    if (q >= 2) wait(&bar.tile_empty[b], ((q >> 1) - 1) & 1);
+    if (q >= 2 && !failed) failed = !mbar_wait_inline(&bar.tile_empty[b], ((q >> 1) - 1) & 1, a.err);
     if (failed) return;  // nothing more is copied
     fillm[q & 3] = fill;
     mx_issue_copies(a, plan, fill, blk, sT + b * MX_TILE, &rec[q & 3], &bar.tile_full[b]);
@@ -2256,8 +2282,8 @@ __global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constan
   // (otherwise the warps have waited for all of them)
   if (failed)
     for (int b = 0; b < 2; b++) {
-      mbar_wait_inline(&bar.tile_full[b], 0, a.err);
-      mbar_wait_inline(&bar.tile_full[b], 1, a.err);
+      mbar_wait_warp<false>(&bar.tile_full[b], 0, a.err);
+      mbar_wait_warp<false>(&bar.tile_full[b], 1, a.err);
     }
 }
 
