@@ -512,8 +512,8 @@ def main():
     ms = ev0.elapsed_time(ev1)
     launches = solver.launch_count()
     # mean stage-kernel launch duration in the timed region itself: the
-    # replayed graph's own event nodes bracket each step's two stage launches
-    # (ghost pre-pass included) on the handle's stream
+    # time-step kernels before and after each step's two stage launches read
+    # the device's clock (ghost pre-pass included)
     stage_ms = solver.timings()[bats.BATS_PHASE_STAGE]
     stage_total_ms = solver.timings()[bats.BATS_PHASE_TOTAL]
     if world > 1:

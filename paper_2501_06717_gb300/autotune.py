@@ -1,7 +1,7 @@
 """Launch autotuner for the fused stage kernel.
 
-Times a few steps per candidate launch form on the live handle (CUDA events
-inside the library bracket the stage kernels) and keeps the fastest:
+Times a few steps per candidate launch form on the live handle (the library's
+own time of the stages) and keeps the fastest:
   persistent     0: one CTA per work item; 1: SMs x CTAs-per-SM CTAs loop
                  over the work items
   blocks_per_cta blocks per work item (consecutive blocks in leaf order, which
@@ -47,7 +47,7 @@ def autotune(solver, cfl, steps=2, candidates=None, use_graph=1, stagings=None):
         if st is not None:
             solver.set_staging(st)
         for cand in candidates or DEFAULT_CANDIDATES:
-            solver.set_launch(cand[0], cand[1], cand[2], 0)  # eager launches: per-stage events
+            solver.set_launch(cand[0], cand[1], cand[2], 0)  # eager launches
             solver.step(1, cfl)
             solver.step(steps, cfl)
             ms = solver.timings()[B.BATS_PHASE_STAGE] / steps

@@ -41,7 +41,8 @@ cudaError_t launch_cfl_dt(bool mixed, const double* U, const float* Wt, const Gr
                           const BlockDev* blocks, const PhysDev& ph, int b0, int nb, unsigned long long* smax,
                           double* dtc, double cfl, cudaStream_t st);
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
-                      unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st);
+                      unsigned long long* smax, unsigned long long* smax_next, unsigned long long* stage_ns,
+                      bool first_step, cudaStream_t st);
 cudaError_t launch_debug_fill(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st);
 cudaError_t launch_debug_fill_w(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st);
 cudaError_t launch_debug_fill_mx(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st);
@@ -77,6 +78,8 @@ struct bats {
   float *W = nullptr, *W1 = nullptr;
   double *dt = nullptr, *t = nullptr;
   unsigned long long *smax = nullptr, *smax_next = nullptr;
+  // error bits, first bad block, fallbacks, -, then (64 bits) the stages' time of
+  // the last call in ns
   int32_t* errw = nullptr;
   double* staging = nullptr;
   size_t staging_n = 0;
@@ -102,8 +105,6 @@ struct bats {
   int stage_tma = 1;
   int occ[2] = {1, 1};
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  std::vector<cudaEvent_t> stage_ev;   // pairs around the two stage launches of each step
-  int timed_steps = 0;
   double ms_last[BATS_NUM_PHASES] = {0, 0, 0};
   long long launches = 0;
   long long fallbacks = 0;  // learned block-stages recomputed with the plain flux
@@ -111,7 +112,6 @@ struct bats {
   int graph_n = -1;
   double graph_cfl = 0, graph_dt = 0;
   long long graph_launches = 0;
-  int graph_timed = 0;                 // steps whose stage events the graph records
   // learned form
   bool learned_requested = false, learned = false;
   bool learned_last_only = false;  // the correction in the last stage of a step only
@@ -433,8 +433,6 @@ void free_all(bats_t* h) {
   cudaFree(h->Yb);
   if (h->ev0) cudaEventDestroy(h->ev0);
   if (h->ev1) cudaEventDestroy(h->ev1);
-  for (cudaEvent_t e : h->stage_ev) cudaEventDestroy(e);
-  h->stage_ev.clear();
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   h->stream = nullptr;
 }
@@ -580,38 +578,14 @@ int launch_local_dt(bats_t* h, double* dtc, double cfl) {
   return BATS_OK;
 }
 
-// Timed steps of a call: an event node between two kernels of a graph costs about
-// 4 us, so all 100 steps of 120 blocks took 4.0 ms with theirs and 3.0 ms without.
-constexpr int kMaxTimedSteps = 8;
-
-int ensure_stage_events(bats_t* h, int n) {
-  int want = 2 * std::min(n, kMaxTimedSteps);
-  while (static_cast<int>(h->stage_ev.size()) < want) {
-    cudaEvent_t e;
-    CK(h, cudaEventCreate(&e));
-    h->stage_ev.push_back(e);
-  }
-  return BATS_OK;
-}
-
-// Enqueue n steps (no synchronisation).  The stage launches of each of the
-// first kMaxTimedSteps steps are bracketed by an event pair: recorded on the
-// stream (timed) or, while a CUDA graph is captured (captured), as event
-// nodes of the graph, which its every replay records.
-int enqueue_steps(bats_t* h, int n, double cfl, double fixed_dt, bool timed, bool captured = false) {
+// Enqueue n steps (no synchronisation).  The time-step kernels around each step's
+// stages add up the stages' time.
+int enqueue_steps(bats_t* h, int n, double cfl, double fixed_dt) {
   const bool mixed = h->ph.precision == BATS_MIXED;
   const bool ssp = h->ph.rk == BATS_RK_SSP2;
   const bool euler = h->ph.rk == BATS_RK_EULER;
   const bool lts = h->local_dt && cfl > 0.0;
-  if (timed) {
-    int rc0 = ensure_stage_events(h, n);
-    if (rc0) return rc0;
-  }
-  h->timed_steps = (timed || captured) ? std::min(n, kMaxTimedSteps) : 0;
-  const int ntimed = h->timed_steps;
-  auto record = [&](cudaEvent_t ev) {
-    return captured ? cudaEventRecordWithFlags(ev, h->stream, cudaEventRecordExternal) : cudaEventRecord(ev, h->stream);
-  };
+  unsigned long long* const stage_ns = reinterpret_cast<unsigned long long*>(h->errw + 4);
   if (lts && n > 0) {
     // every cell's dt from the current state (later steps take it from the
     // last stage of the step before)
@@ -625,9 +599,8 @@ int enqueue_steps(bats_t* h, int n, double cfl, double fixed_dt, bool timed, boo
   float* Wcur = h->W;
   float* Woth = h->W1;
   for (int s = 0; s < n; s++) {
-    CK(h, launch_dt(h->ngrids, 0, cfl, fixed_dt, h->dt, h->t, h->smax, h->smax_next, h->stream));
+    CK(h, launch_dt(h->ngrids, 0, cfl, fixed_dt, h->dt, h->t, h->smax, h->smax_next, stage_ns, s == 0, h->stream));
     h->launches++;
-    if (s < ntimed) CK(h, record(h->stage_ev[2 * s]));
     StageArgs a = base_args(h);
     a.dtc = lts ? h->dtc : nullptr;
     a.cfl = cfl;
@@ -673,8 +646,7 @@ int enqueue_steps(bats_t* h, int n, double cfl, double fixed_dt, bool timed, boo
       rc = launch_stage(h, a);
       if (rc) return rc;
     }
-    if (s < ntimed) CK(h, record(h->stage_ev[2 * s + 1]));
-    CK(h, launch_dt(h->ngrids, 1, cfl, fixed_dt, h->dt, h->t, h->smax, h->smax_next, h->stream));
+    CK(h, launch_dt(h->ngrids, 1, cfl, fixed_dt, h->dt, h->t, h->smax, h->smax_next, stage_ns, false, h->stream));
     h->launches++;
   }
   if (Ucur != h->U) {
@@ -707,12 +679,10 @@ int run_steps(bats_t* h, int n, double cfl, double fixed_dt, double* t_out) {
   if (h->use_graph && n > 0) {
     if (!h->graph || h->graph_n != n || h->graph_cfl != cfl || h->graph_dt != fixed_dt) {
       if (h->graph) { cudaGraphExecDestroy(h->graph); h->graph = nullptr; }
-      // the events the graph's event nodes record exist before the capture
-      if (int rc0 = ensure_stage_events(h, n)) return rc0;
       cudaGraph_t g;
       CK(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
       h->launches = 0;
-      int rc = enqueue_steps(h, n, cfl, fixed_dt, false, true);
+      int rc = enqueue_steps(h, n, cfl, fixed_dt);
       cudaError_t e = cudaStreamEndCapture(h->stream, &g);
       if (rc) return rc;
       if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
@@ -723,32 +693,25 @@ int run_steps(bats_t* h, int n, double cfl, double fixed_dt, double* t_out) {
       h->graph_cfl = cfl;
       h->graph_dt = fixed_dt;
       h->graph_launches = h->launches;
-      h->graph_timed = h->timed_steps;
     }
     CK(h, cudaGraphLaunch(h->graph, h->stream));
     h->launches = h->graph_launches;
-    h->timed_steps = h->graph_timed;
   } else {
-    int rc = enqueue_steps(h, n, cfl, fixed_dt, true);
+    int rc = enqueue_steps(h, n, cfl, fixed_dt);
     if (rc) return rc;
   }
   CK(h, cudaEventRecord(h->ev1, h->stream));
-  int32_t ew[3];
+  int32_t ew[6];
   CK(h, cudaMemcpyAsync(ew, h->errw, sizeof(ew), cudaMemcpyDeviceToHost, h->stream));
   CK(h, cudaStreamSynchronize(h->stream));
   h->fallbacks += ew[2];
   float ms = 0.f;
   CK(h, cudaEventElapsedTime(&ms, h->ev0, h->ev1));
-  double stage_ms = 0.0;
-  for (int s = 0; s < h->timed_steps && n > 0; s++) {
-    float m = 0.f;
-    CK(h, cudaEventElapsedTime(&m, h->stage_ev[2 * s], h->stage_ev[2 * s + 1]));
-    stage_ms += m;
-  }
-  if (h->timed_steps > 0 && n > h->timed_steps) stage_ms *= static_cast<double>(n) / h->timed_steps;
-  stage_ms = std::min(stage_ms, static_cast<double>(ms));  // (scaled from the first steps)
-  h->ms_last[BATS_PHASE_STAGE] = h->timed_steps > 0 ? stage_ms : -1.0;
-  h->ms_last[BATS_PHASE_DT] = h->timed_steps > 0 ? ms - stage_ms : -1.0;
+  unsigned long long stage_ns = 0;
+  std::memcpy(&stage_ns, ew + 4, sizeof(stage_ns));
+  const double stage_ms = 1e-6 * static_cast<double>(stage_ns);
+  h->ms_last[BATS_PHASE_STAGE] = n > 0 ? stage_ms : -1.0;
+  h->ms_last[BATS_PHASE_DT] = n > 0 ? ms - stage_ms : -1.0;
   h->ms_last[BATS_PHASE_TOTAL] = ms;
   if (t_out) CK(h, cudaMemcpy(t_out, h->t, sizeof(double), cudaMemcpyDeviceToHost));
   if (int rc = index_check(h)) return rc;
@@ -884,7 +847,7 @@ int bats_create(const bats_grid_desc* grids, int n_grids, const bats_physics* ph
       (rc = dev_alloc(h, &h->levmap_d, h->levmap_h.size())) || (rc = dev_alloc(h, &h->U, nstate)) ||
       (rc = dev_alloc(h, &h->U1, nstate)) || (rc = dev_alloc(h, &h->dt, h->ngrids)) ||
       (rc = dev_alloc(h, &h->t, h->ngrids)) || (rc = dev_alloc(h, &h->smax, h->ngrids)) ||
-      (rc = dev_alloc(h, &h->smax_next, h->ngrids)) || (rc = dev_alloc(h, &h->errw, 3)) ||
+      (rc = dev_alloc(h, &h->smax_next, h->ngrids)) || (rc = dev_alloc(h, &h->errw, 6)) ||
       (rc = dev_alloc(h, &h->staging, h->staging_n))) {
     free_all(h);
     g_create_error = h->err;
@@ -1299,7 +1262,7 @@ int bats_debug_face_data(bats_t* h, int grid, int stage_input, double dt, float*
   const double* Uin = h->U;
   const float* Win = h->W;
   if (e == cudaSuccess && stage_input) {
-    e = launch_dt(h->ngrids, 0, -1.0, dt, h->dt, h->t, h->smax, h->smax_next, h->stream);
+    e = launch_dt(h->ngrids, 0, -1.0, dt, h->dt, h->t, h->smax, h->smax_next, nullptr, false, h->stream);
     StageArgs s1 = a;
     s1.Uin = h->U;
     s1.Ubase = h->U;

@@ -33,7 +33,8 @@ cudaError_t launch_store_state(const double* U, double* ext, int64_t ext_off, co
                                const BlockDev* blocks, int b0, int nb, cudaStream_t st);
 cudaError_t launch_init_grid_states(GridDev* grids, int ngrids, double inv_gm1, double gm1, cudaStream_t st);
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
-                      unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st);
+                      unsigned long long* smax, unsigned long long* smax_next, unsigned long long* stage_ns,
+                      bool first_step, cudaStream_t st);
 cudaError_t read_index_flag(int32_t* out);
 }  // namespace batsk
 
@@ -379,7 +380,7 @@ extern "C" int bats_step_noalloc(const bats_grid_desc* grid, const bats_physics*
   double* Ucur = Ui;
   double* Uoth = U1;
   for (int s = 0; s < steps; s++) {
-    NA_CK(launch_dt(1, 0, c, dt, dtw, tw, smax, smax_next, st));
+    NA_CK(launch_dt(1, 0, c, dt, dtw, tw, smax, smax_next, nullptr, false, st));
     if (euler) {
       a.Uin = Ucur;
       a.Ubase = Ucur;
@@ -388,7 +389,7 @@ extern "C" int bats_step_noalloc(const bats_grid_desc* grid, const bats_physics*
       a.last = 1;
       a.beta = 1.0;
       NA_CK(launch_stage_kernel(false, nb, st, a));
-      NA_CK(launch_dt(1, 1, c, dt, dtw, tw, smax, smax_next, st));
+      NA_CK(launch_dt(1, 1, c, dt, dtw, tw, smax, smax_next, nullptr, false, st));
       double* tmp = Ucur;
       Ucur = Uoth;
       Uoth = tmp;
@@ -408,7 +409,7 @@ extern "C" int bats_step_noalloc(const bats_grid_desc* grid, const bats_physics*
     a.last = 1;
     a.beta = 1.0;
     NA_CK(launch_stage_kernel(false, nb, st, a));
-    NA_CK(launch_dt(1, 1, c, dt, dtw, tw, smax, smax_next, st));
+    NA_CK(launch_dt(1, 1, c, dt, dtw, tw, smax, smax_next, nullptr, false, st));
   }
   if (Ucur != Ui) NA_CK(cudaMemcpyAsync(Ui, Ucur, bytes, cudaMemcpyDeviceToDevice, st));
   // block-major -> caller layout (host destinations staged through U1)

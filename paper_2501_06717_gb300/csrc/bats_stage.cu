@@ -455,10 +455,16 @@ __global__ void __launch_bounds__(64) k_reflux(const StageArgs a, const RefluxTa
 // Per-grid time-step bookkeeping.
 //  mode 0 (before a step): dt = cfl > 0 ? cfl / smax : fixed_dt; smax_next = 0
 //  mode 1 (after a step):  t += dt; smax = smax_next
+// stage_ns (nullable): the time between the two, the stages' time, summed over the
+// steps of a call (from 0 with first_step), by the device's clock (32 ns): event
+// nodes around each step's stages cost a graph about 8 us a step.
 __global__ void k_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
-                     unsigned long long* smax, unsigned long long* smax_next) {
+                     unsigned long long* smax, unsigned long long* smax_next, unsigned long long* stage_ns,
+                     bool first_step) {
   pdl_begin();
   int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const bool clocked = g == 0 && stage_ns;
+  if (clocked && mode == 1) *stage_ns += globaltimer();
   if (g >= ngrids) return;
   if (mode == 0) {
     double s = __longlong_as_double(static_cast<long long>(smax[g]));
@@ -468,6 +474,7 @@ __global__ void k_dt(int ngrids, int mode, double cfl, double fixed_dt, double* 
     t[g] += dt[g];
     smax[g] = smax_next[g];
   }
+  if (clocked && mode == 0) *stage_ns = (first_step ? 0ull : *stage_ns) - globaltimer();
 }
 
 // Padded tiles [8][nb][12][12][12] (external layout) of the shared-memory
@@ -698,8 +705,10 @@ cudaError_t launch_reflux(bool mixed, const StageArgs& a, const RefluxTask* task
   return cudaGetLastError();
 }
 cudaError_t launch_dt(int ngrids, int mode, double cfl, double fixed_dt, double* dt, double* t,
-                      unsigned long long* smax, unsigned long long* smax_next, cudaStream_t st) {
-  return launch_pdl(k_dt, (ngrids + 127) / 128, 128, 0, st, ngrids, mode, cfl, fixed_dt, dt, t, smax, smax_next);
+                      unsigned long long* smax, unsigned long long* smax_next, unsigned long long* stage_ns,
+                      bool first_step, cudaStream_t st) {
+  return launch_pdl(k_dt, (ngrids + 127) / 128, 128, 0, st, ngrids, mode, cfl, fixed_dt, dt, t, smax, smax_next,
+                    stage_ns, first_step);
 }
 cudaError_t launch_debug_fill(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st) {
   k_debug_fill<<<nb, 256, sizeof(double) * (NV * NTILE + 3 * 128 * NV), st>>>(a, b0, nb, T);
