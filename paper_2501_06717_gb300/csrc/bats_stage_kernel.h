@@ -270,8 +270,10 @@ __device__ __forceinline__ void b0_at(const PhysDev& ph, const R x[3], R B0[3]) 
     R r2 = x[0] * x[0] + x[1] * x[1] + x[2] * x[2];
     R inv_r5;
     if constexpr (std::is_same<R, double>::value) {
-      const double ir = div_sqrt64(1.0, r2), ir2 = ir * ir;
-      inv_r5 = ir2 * ir2 * ir;
+      // at r = 0 a reciprocal of 0: the field there is NaN, as in FP32, and a cell
+      // or face that needs it makes the step non-physical.  (r2^2 r before the
+      // reciprocal: half the rounding errors of the fifth power of 1/r.)
+      inv_r5 = rcp64(r2 * r2 * sqrt64(r2));
     } else {
       R r = Ops<R>::sqrt_(r2);
       inv_r5 = Ops<R>::div_(R(1), r2 * r2 * r);
