@@ -282,6 +282,13 @@ int bats_get_fallbacks(bats_t* h, long long* n);
  * the compiler's conversions.  Allocates and frees its own device buffers. */
 int bats_debug_check_conversions(const float* f, const double* d, int n, double* f2d_out, float* d2f_out);
 
+/* Self-check of the FP64 form's operations made from the hardware's estimates:
+ * in[4][n] = a, x, b, c (host); out[5][n] = 1/x, sqrt(x), a/sqrt(x), the
+ * velocity a/x of the primitive recovery, and the fast magnetosonic speed for
+ * half the sound term gamma p / 2 = a, density x, total B^2 = b and squared
+ * normal field c.  Allocates and frees its own device buffers. */
+int bats_debug_fp64_ops(const double* in, int n, double* out);
+
 /* Self-check of the network's activation (the learned correction's GELU,
  * tanh form, Hendrycks & Gimpel): y[i] = the kernels' GELU of x[i] as they
  * compute it for the hidden activations -- two values at a time in packed

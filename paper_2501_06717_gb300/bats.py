@@ -115,6 +115,7 @@ def lib():
     L.bats_get_launch_count.argtypes = [vp, ctypes.POINTER(ctypes.c_longlong)]
     L.bats_get_fallbacks.argtypes = [vp, ctypes.POINTER(ctypes.c_longlong)]
     L.bats_debug_check_conversions.argtypes = [vp, vp, ctypes.c_int, vp, vp]
+    L.bats_debug_fp64_ops.argtypes = [vp, ctypes.c_int, vp]
     L.bats_debug_gelu.argtypes = [vp, ctypes.c_int, ctypes.c_int, vp]
     L.bats_set_mlp.argtypes = [vp, vp]
     L.bats_debug_face_data.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_double, vp, vp, ctypes.c_size_t]
@@ -353,6 +354,19 @@ def bats_debug_check_conversions(f, d):
     if rc != BATS_OK:
         raise BatsError(rc, "conversion check failed")
     return o1, o2
+
+
+def bats_debug_fp64_ops(a, x, b=None, c=None):
+    """The FP64 form's (1/x, sqrt(x), a/sqrt(x), a/x, fast speed(a, x, b, c))."""
+    x = np.asarray(x, dtype=np.float64)
+    z = np.zeros_like(x)
+    rows = np.ascontiguousarray([np.asarray(a, dtype=np.float64), x, z if b is None else b, z if c is None else c],
+                                dtype=np.float64)
+    out = np.zeros((5, x.size))
+    rc = lib().bats_debug_fp64_ops(rows.ctypes.data, int(x.size), out.ctypes.data)
+    if rc != BATS_OK:
+        raise BatsError(rc, "FP64 operation check failed")
+    return tuple(out)
 
 
 def bats_debug_gelu(x, variant=0):

@@ -47,6 +47,7 @@ cudaError_t launch_debug_fill(const StageArgs& a, int b0, int nb, double* T, cud
 cudaError_t launch_debug_fill_w(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st);
 cudaError_t launch_debug_fill_mx(const StageArgs& a, int b0, int nb, double* T, cudaStream_t st);
 cudaError_t launch_check_conversions(const float* f, const double* d, int n, double* f2d_out, float* d2f_out);
+cudaError_t launch_debug_fp64_ops(const double* in, int n, double* out);
 cudaError_t launch_fp64_fma_rate(double* out, int ctas, int iters, cudaStream_t st);
 cudaError_t read_index_flag(int32_t* out);
 cudaError_t launch_debug_wait_timeout(int32_t* err, cudaStream_t st);
@@ -1339,6 +1340,20 @@ int bats_debug_check_conversions(const float* f, const double* d, int n, double*
   cudaFree(dd);
   cudaFree(of2d);
   cudaFree(od2f);
+  return e == cudaSuccess ? BATS_OK : BATS_ERR_CUDA;
+}
+
+int bats_debug_fp64_ops(const double* in, int n, double* out) {
+  if (!in || n <= 0 || !out) return BATS_ERR_INVALID_ARG;
+  const size_t row = static_cast<size_t>(n) * sizeof(double);
+  double *di = nullptr, *dout = nullptr;
+  cudaError_t e = cudaMalloc(&di, 4 * row);
+  if (e == cudaSuccess) e = cudaMalloc(&dout, 5 * row);
+  if (e == cudaSuccess) e = cudaMemcpy(di, in, 4 * row, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = launch_debug_fp64_ops(di, n, dout);
+  if (e == cudaSuccess) e = cudaMemcpy(out, dout, 5 * row, cudaMemcpyDeviceToHost);
+  cudaFree(di);
+  cudaFree(dout);
   return e == cudaSuccess ? BATS_OK : BATS_ERR_CUDA;
 }
 

@@ -579,6 +579,23 @@ __global__ void k_check_conversions(const float* f, const double* d, int n, doub
   d2f_out[i] = d2f_int(d[i]);
 }
 
+// The FP64 form's operations on n values each of a, x, b, c: 1/x, sqrt(x),
+// a/sqrt(x), the velocity a/x of prim64, and the fast speed for half the sound
+// term a, density x, B^2 = b and squared normal field c; out[5][n].
+__global__ void k_debug_fp64_ops(const double* in, int n, double* out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double a = in[i], x = in[n + i], b = in[2 * n + i], c = in[3 * n + i];
+  const double U[8] = {x, a, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  double W[8];
+  prim64(U, 1.0, W);
+  out[i] = rcp64(x);
+  out[n + i] = sqrt64(x);
+  out[2 * n + i] = div_sqrt64(a, x);
+  out[3 * n + i] = W[1];
+  out[4 * n + i] = fast_speed64(a, b, c, x);
+}
+
 // ---------------------------------------------------------------------------
 // Host-side launchers (kernel stubs stay in this translation unit).
 
@@ -788,6 +805,11 @@ __global__ void __launch_bounds__(256) k_fp64_fma_rate(double* out, int iters, d
 }
 cudaError_t launch_fp64_fma_rate(double* out, int ctas, int iters, cudaStream_t st) {
   k_fp64_fma_rate<<<ctas, 256, 0, st>>>(out, iters, 0.9999999, 1e-7, -1.0);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_debug_fp64_ops(const double* in, int n, double* out) {
+  k_debug_fp64_ops<<<(n + 255) / 256, 256>>>(in, n, out);
   return cudaGetLastError();
 }
 

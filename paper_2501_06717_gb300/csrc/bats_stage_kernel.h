@@ -183,8 +183,9 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // one third-order Newton step (Householder's method, order 2: the error cubed):
 // with e = 1 - x y,      1/x       = y (1 + e + e^2) + O(e^3);
 // with r = 1 - x y^2,    1/sqrt(x) = y (1 + r/2 + 3 r^2 / 8) + O(r^3).
-// The last operation is an FMA onto the leading term, so the results are within
-// about one unit in the last place.  GB300 issues 2 FP64 operations per clock
+// The last operation is an FMA onto the leading term, so 1/x is off by little more
+// than its own rounding (u = 2^-53 relative), sqrt(x) by 1.5 u (half of the
+// rounding of x y) and a/sqrt(x) by 2.5 u (that of a y too).  GB300 issues 2 FP64 operations per clock
 // and SM: these take 3 and 5 of them where the general division and square root
 // take several times as many, and a face has two speeds of two roots each.
 __device__ __forceinline__ double rcp64(double x) {
@@ -292,8 +293,14 @@ __device__ __forceinline__ void b0_at(const PhysDev& ph, const R x[3], R B0[3]) 
 
 // Primitive recovery in FP64 (Eq. 5): u = m/rho, p = (gamma-1)(e1 - m.u/2 - B1.B1/2).
 __device__ __forceinline__ void prim64(const double U[8], double gm1, double W[8]) {
+  // U / rho rounded like a division: the quotient by 1 / rho, then its (exact)
+  // remainder.  Without the remainder the residuals were up to 0.5 % further from
+  // an 80-bit evaluation than with divisions, with it they are 1 to 2 % nearer.
   const double rinv = rcp64(U[0]);
-  const double ux = U[1] * rinv, uy = U[2] * rinv, uz = U[3] * rinv;
+  double ux = U[1] * rinv, uy = U[2] * rinv, uz = U[3] * rinv;
+  ux = fma(fma(-U[0], ux, U[1]), rinv, ux);
+  uy = fma(fma(-U[0], uy, U[2]), rinv, uy);
+  uz = fma(fma(-U[0], uz, U[3]), rinv, uz);
   const double ke2 = fma(U[3], uz, fma(U[2], uy, U[1] * ux));
   const double me2 = fma(U[6], U[6], fma(U[5], U[5], U[4] * U[4]));
   W[0] = U[0]; W[1] = ux; W[2] = uy; W[3] = uz;
@@ -1170,7 +1177,7 @@ __device__ __forceinline__ void side64(const double w[8], const double B0[3], do
   cf = fast_speed64(hgamma * p, tsq, tt0, rho);
   const double ub = fma(u2, b2, fma(u1, b1, u0 * b0));
   double pt = fma(0.5, bsq, p);
-  if constexpr (HAS_B0) pt = fma(B0[2], b2, fma(B0[1], b1, fma(B0[0], b0, pt)));
+  if constexpr (HAS_B0) pt += fma(B0[2], b2, fma(B0[1], b1, B0[0] * b0));
   U[0] = rho;
   U[1] = rho * u0;
   U[2] = rho * u1;
@@ -1180,13 +1187,16 @@ __device__ __forceinline__ void side64(const double w[8], const double B0[3], do
   U[6] = b2;
   U[7] = fma(p, inv_gm1, 0.5 * fma(U[3], u2, fma(U[2], u1, fma(U[1], u0, bsq))));
   F[0] = U[1];
-  F[1] = fma(U[1], u0, fma(-b0, T0, pt));
-  F[2] = fma(U[2], u0, -(b1 * T0));
-  F[3] = fma(U[3], u0, -(b2 * T0));
+  // B1 B_n + B0 B1_n (with a background field summed first, so that the flux is
+  // rounded once)
   if constexpr (HAS_B0) {
-    F[1] = fma(-B0[0], b0, F[1]);
-    F[2] = fma(-B0[1], b0, F[2]);
-    F[3] = fma(-B0[2], b0, F[3]);
+    F[1] = fma(U[1], u0, fma(-b0, T0 + B0[0], pt));
+    F[2] = fma(U[2], u0, -fma(b1, T0, B0[1] * b0));
+    F[3] = fma(U[3], u0, -fma(b2, T0, B0[2] * b0));
+  } else {
+    F[1] = fma(U[1], u0, fma(-b0, T0, pt));
+    F[2] = fma(U[2], u0, -(b1 * T0));
+    F[3] = fma(U[3], u0, -(b2 * T0));
   }
   F[4] = 0.0;
   F[5] = fma(u0, T1, -(T0 * u1));
