@@ -178,6 +178,10 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 }
 
 // ---------------------------------------------------------------------------
+// Divisions and roots of numbers far from one, by the general operations (calls,
+// so that the branches to them keep no registers).
+static __device__ __noinline__ double div_far(double a, double b) { return a / b; }
+static __device__ __noinline__ double sqrt_far(double x) { return sqrt(x); }
 // FP64 reciprocal and square roots from the hardware's estimates (PTX
 // rcp/rsqrt.approx.ftz.f64, about 20 bits, issued off the FP64 pipe) refined by
 // one third-order Newton step (Householder's method, order 2: the error cubed):
@@ -188,7 +192,14 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 // rounding of x y) and a/sqrt(x) by 2.5 u (that of a y too).  GB300 issues 2 FP64 operations per clock
 // and SM: these take 3 and 5 of them where the general division and square root
 // take several times as many, and a face has two speeds of two roots each.
+// rcp64 takes any x (its estimate is flushed to 0 or infinity where x or 1/x is
+// not a normal number: there the division); sqrt64 takes 0 and positive normal x,
+// div_sqrt64 positive normal x.
+__device__ __forceinline__ bool rcp_normal(double x) {
+  return (static_cast<uint32_t>(__double2hiint(x)) & 0x7fffffffu) - 0x00100000u < 0x7fd00000u - 0x00100000u;
+}
 __device__ __forceinline__ double rcp64(double x) {
+  if (!rcp_normal(x)) return div_far(1.0, x);
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
@@ -216,9 +227,22 @@ __device__ __forceinline__ double div_sqrt64(double a, double x) {
 // normal field and rho:
 //   c_f^2 = (G + sqrt(G^2 - gamma p B_n^2)) / rho,  G = (gamma p + B^2) / 2,
 // the usual form with 1/rho taken out of both roots, which leaves no division
-// (c_f = Q / sqrt(Q rho)).
+// (c_f = Q / sqrt(Q rho)).  Its square G^2 and product Q rho are normal numbers
+// for G and rho in 2^-450 .. 2^450; everything else (a scale where only the
+// speeds are near one, negative, NaN) takes the usual form itself.  The test and
+// the code around it cost the FP64 form 0.6 to 1.2 %.
+__device__ __forceinline__ bool mid_range(double x) {
+  return static_cast<uint32_t>(__double2hiint(x)) - (573u << 20) < (900u << 20);
+}
+static __device__ __noinline__ double fast_speed_far(double gp, double bsq, double bn2, double rho) {
+  const double a2 = gp / rho, s = a2 + bsq / rho;
+  double disc = s * s - 4.0 * a2 * (bn2 / rho);
+  disc = disc < 0.0 ? 0.0 : disc;
+  return sqrt(0.5 * (s + sqrt(disc)));
+}
 __device__ __forceinline__ double fast_speed64(double gph, double bsq, double bn2, double rho) {
   const double G = fma(0.5, bsq, gph);
+  if (!(mid_range(G) && mid_range(rho))) return fast_speed_far(2.0 * gph, bsq, bn2, rho);
   double D = fma(-2.0, gph * bn2, G * G);
   D = __double2hiint(D) < 0 ? 0.0 : D;
   const double Q = G + sqrt64(D);
@@ -296,11 +320,20 @@ __device__ __forceinline__ void prim64(const double U[8], double gm1, double W[8
   // U / rho rounded like a division: the quotient by 1 / rho, then its (exact)
   // remainder.  Without the remainder the residuals were up to 0.5 % further from
   // an 80-bit evaluation than with divisions, with it they are 1 to 2 % nearer.
-  const double rinv = rcp64(U[0]);
-  double ux = U[1] * rinv, uy = U[2] * rinv, uz = U[3] * rinv;
-  ux = fma(fma(-U[0], ux, U[1]), rinv, ux);
-  uy = fma(fma(-U[0], uy, U[2]), rinv, uy);
-  uz = fma(fma(-U[0], uz, U[3]), rinv, uz);
+  double ux, uy, uz;
+  if (rcp_normal(U[0])) {
+    const double rinv = rcp64(U[0]);
+    ux = U[1] * rinv;
+    uy = U[2] * rinv;
+    uz = U[3] * rinv;
+    ux = fma(fma(-U[0], ux, U[1]), rinv, ux);
+    uy = fma(fma(-U[0], uy, U[2]), rinv, uy);
+    uz = fma(fma(-U[0], uz, U[3]), rinv, uz);
+  } else {
+    ux = div_far(U[1], U[0]);
+    uy = div_far(U[2], U[0]);
+    uz = div_far(U[3], U[0]);
+  }
   const double ke2 = fma(U[3], uz, fma(U[2], uy, U[1] * ux));
   const double me2 = fma(U[6], U[6], fma(U[5], U[5], U[4] * U[4]));
   W[0] = U[0]; W[1] = ux; W[2] = uy; W[3] = uz;
@@ -435,13 +468,21 @@ __device__ __forceinline__ double minmod_d(double a, double b) {
   return same ? __longlong_as_double(r) : 0.0;
 }
 // Comparisons of doubles on bit patterns (a comparison shares the FP64 pipe,
-// which bounds the FP64 form): the order of non-NaN values as signed integers.
+// which bounds the FP64 form): the order of non-NaN values as signed integers;
+// max_d is a > b ? a : b and min_d a < b ? a : b (with a NaN, b).
 __device__ __forceinline__ long long order_d(double x) {
   const long long i = __double_as_longlong(x);
   return i ^ ((i >> 63) & 0x7fffffffffffffffll);
 }
-__device__ __forceinline__ double max_d(double a, double b) { return order_d(a) > order_d(b) ? a : b; }
-__device__ __forceinline__ double min_d(double a, double b) { return order_d(a) < order_d(b) ? a : b; }
+__device__ __forceinline__ bool nan_d(double x) {  // (a quiet NaN: the result of an operation)
+  return (static_cast<uint32_t>(__double2hiint(x)) & 0x7fffffffu) > 0x7ff00000u;
+}
+__device__ __forceinline__ double max_d(double a, double b) {
+  return order_d(a) > order_d(b) && !nan_d(a) && !nan_d(b) ? a : b;
+}
+__device__ __forceinline__ double min_d(double a, double b) {
+  return order_d(a) < order_d(b) && !nan_d(a) && !nan_d(b) ? a : b;
+}
 // Validity tests on bit patterns: finite, and finite and > 0.
 __device__ __forceinline__ bool finite_d(double x) {
   return (static_cast<unsigned>(__double2hiint(x)) & 0x7ff00000u) != 0x7ff00000u;
@@ -1219,7 +1260,9 @@ __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[
     // cfR, 0):  F = F_L - S_L/(S_R - S_L) ((F_R - F_L) - S_R (U_R - U_L))
     const double sl = min_d(min_d(wl[1] - cl, wr[1] - cr), 0.0), sr = max_d(max_d(wl[1] + cl, wr[1] + cr), 0.0);
     const double den = sr - sl;
-    const double kk = __double_as_longlong(den) > 0 ? sl * rcp64(den) : 0.0;
+    // den > 0 (not NaN)
+    const bool open = static_cast<unsigned long long>(__double_as_longlong(den)) - 1 < 0x7ff0000000000000ull;
+    const double kk = open ? sl * rcp64(den) : 0.0;
 #pragma unroll
     for (int v = 0; v < NV; v++) {
       const double dU = UR[v] - UL[v];
@@ -1232,7 +1275,14 @@ __device__ __forceinline__ void face_flux64(const double wl[8], const double wr[
       // face states, c^2 = gamma p / rho
       const double um0 = 0.5 * (wl[1] + wr[1]), um1 = 0.5 * (wl[2] + wr[2]), um2 = 0.5 * (wl[3] + wr[3]);
       const double gp = hgamma * (wl[7] + wr[7]), rm = 0.5 * (wl[0] + wr[0]);
-      const double cs = div_sqrt64(gp, gp * rm), ic2 = rm * rcp64(gp);
+      double cs, ic2;
+      if (mid_range(gp) && mid_range(rm)) {
+        cs = div_sqrt64(gp, gp * rm);
+        ic2 = rm * rcp64(gp);
+      } else {
+        cs = sqrt_far(div_far(gp, rm));
+        ic2 = div_far(rm, gp);
+      }
       const double dr = wr[0] - wl[0];
       const double alpha = minmod_d(fma(-(wr[7] - wl[7]), ic2, dr), dr);
       const double q = kk == 0.0 ? 0.0 : kk * sr * alpha * (cs * rcp64(cs + fabs(um0)));
