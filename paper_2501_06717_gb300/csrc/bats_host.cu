@@ -381,6 +381,16 @@ int build_grid(bats_t* h, const bats_grid_desc& d, int gidx, int block0, std::ve
 template <class T>
 int dev_alloc(bats_t* h, T** p, size_t n) {
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(n, 1) * sizeof(T));
+  if (e == cudaErrorMemoryAllocation && h->b0t) {
+    // the stage can do without the table (and no captured graph may keep it)
+    cudaGetLastError();
+    if (h->graph) cudaGraphExecDestroy(h->graph);
+    h->graph = nullptr;
+    cudaStreamSynchronize(h->stream);
+    cudaFree(h->b0t);
+    h->b0t = nullptr;
+    e = cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(n, 1) * sizeof(T));
+  }
   if (e != cudaSuccess) return fail(h, BATS_ERR_OUT_OF_MEMORY, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   return BATS_OK;
 }
@@ -872,13 +882,6 @@ int bats_create(const bats_grid_desc* grids, int n_grids, const bats_physics* ph
     delete h;
     return rc;
   }
-  if (h->ph.b0 != BATS_B0_NONE &&
-      (rc = dev_alloc(h, &h->b0t, static_cast<size_t>(h->nbt) * 7 * NCELL * (h->ph.precision == BATS_MIXED ? 4 : 8)))) {
-    free_all(h);
-    g_create_error = h->err;
-    delete h;
-    return rc;
-  }
   if (h->local_dt && (rc = dev_alloc(h, &h->dtc, static_cast<size_t>(h->nbt) * NCELL))) {
     free_all(h);
     g_create_error = h->err;
@@ -893,6 +896,13 @@ int bats_create(const bats_grid_desc* grids, int n_grids, const bats_physics* ph
       delete h;
       return rc;
     }
+  }
+  // last, because the handle works without it
+  if ((h->ph.b0 == BATS_B0_DIPOLE || h->ph.b0 == BATS_B0_LINEAR) &&
+      cudaMalloc(reinterpret_cast<void**>(&h->b0t),
+                 static_cast<size_t>(h->nbt) * 7 * NCELL * (h->ph.precision == BATS_MIXED ? 4 : 8)) != cudaSuccess) {
+    cudaGetLastError();
+    h->b0t = nullptr;
   }
   e = cudaMemcpyAsync(h->grids_d, h->grids_h.data(), sizeof(GridDev) * h->ngrids, cudaMemcpyHostToDevice, h->stream);
   if (e == cudaSuccess)

@@ -135,7 +135,8 @@ struct StageArgs {
                           // state by the last stage (nullptr: global dt)
   double cfl;             // CFL number for dtc
   const void* b0t;        // background field: per cell B0 at the centre, div B0, curl B0 [block][7][512] in the
-                          // stage's precision, made once per handle (nullptr: evaluated in the kernel)
+                          // stage's precision, made once per handle (nullptr: evaluated in the kernel: a uniform
+                          // field, no room for a table, bats_step_noalloc)
   double* freg;           // refluxing: flux register [slot][64][8] (nullptr: off)
   float* gbuf;            // mixed form: ghost slabs of faces at resolution changes [slot][8][128]
   int32_t nslots;         // slots of freg and gbuf (index checks of the checked build)

@@ -296,7 +296,7 @@ template <class R>
 __global__ void __launch_bounds__(NCELL) k_b0_table(const GridDev* grids, const BlockDev* blocks, const PhysDev ph, R* t) {
   const BlockDev& B = blocks[blockIdx.x];
   R o[7];
-  b0_cell_eval<R>(ph, grids[B.grid], B, threadIdx.x, o);
+  b0_cell_call<R>(ph, grids[B.grid], B, threadIdx.x, o);
 #pragma unroll
   for (int k = 0; k < 7; k++) t[(static_cast<int64_t>(blockIdx.x) * 7 + k) * NCELL + threadIdx.x] = o[k];
 }

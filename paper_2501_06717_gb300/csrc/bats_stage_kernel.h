@@ -1148,23 +1148,34 @@ __device__ __forceinline__ void b0_cell_eval(const PhysDev& ph, const GridDev& G
   o[5] = (zp[0] - zm[0]) * idx2 - (xp[2] - xm[2]) * idx0;
   o[6] = (xp[1] - xm[1]) * idx0 - (yp[0] - ym[0]) * idx1;
 }
-static __device__ __noinline__ void b0_cell_eval64(const PhysDev& ph, const GridDev& G, const BlockDev& B, int c,
-                                                   double o[7]) {
-  b0_cell_eval<double>(ph, G, B, c, o);
+template <class R>
+static __device__ __noinline__ void b0_cell_call(const PhysDev& ph, const GridDev& G, const BlockDev& B, int c, R o[7]) {
+  if (ph.b0 == B0_UNIFORM) {  // (the same values: differences of equal face values)
+    for (int k = 0; k < 7; k++) o[k] = k < 3 ? R(ph.b0p[k]) : R(0);
+    return;
+  }
+  b0_cell_eval<R>(ph, G, B, c, o);
 }
-// The same from the handle's table: seven coalesced loads instead of seven
-// evaluations of the field (a dipole: two roots and a division each):
-// magnetosphere, 3,872 blocks, mixed 10 steps 6.56 -> 4.97 ms, FP64 2 steps 21.3
-// -> 16.5 ms, for 28 or 56 bytes per cell of reads and of memory.  The FP64
-// form without a table (bats_step_noalloc keeps none) evaluates.
+// The same from the handle's table where it has one (a linear or dipole field and
+// room for it): seven coalesced loads instead of seven evaluations of the field (a
+// dipole: two roots and a division each), for 28 or 56 bytes per cell of reads and
+// of memory.  2,344 blocks (dipole: 1,728) with the table and without: linear
+// 1.48 and 3.18 ms (4 steps, mixed), 8.8 and 9.7 (2 steps, FP64); dipole 0.80 and
+// 1.24, 6.9 and 8.4.  A uniform field's three constants and four zeros need none:
+// 0.97 ms with them and with a table, FP64 8.4 both ways; in line in the mixed
+// form (a call: 1.02 ms), by the call in FP64 (in line the magnetosphere's steps
+// take 17.2 instead of 16.9 ms).
 template <class R>
 __device__ __forceinline__ void b0_cell(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk, int c, R o[7]) {
-  if (std::is_same<R, float>::value || a.b0t) {
-    const R* t = static_cast<const R*>(a.b0t) + static_cast<int64_t>(blk) * (7 * NCELL) + c;
+  if (a.b0t) {
+    const R* t = static_cast<const R*>(a.b0t) + chk(blk, 0, a.nblocks) * (7 * NCELL) + chki(c, 0, NCELL);
 #pragma unroll
     for (int k = 0; k < 7; k++) o[k] = t[k * NCELL];
+  } else if (std::is_same<R, float>::value && a.ph.b0 == B0_UNIFORM) {
+#pragma unroll
+    for (int k = 0; k < 7; k++) o[k] = k < 3 ? R(a.ph.b0p[k]) : R(0);
   } else {
-    if constexpr (std::is_same<R, double>::value) b0_cell_eval64(a.ph, G, B, c, o);
+    b0_cell_call<R>(a.ph, G, B, c, o);
   }
 }
 
