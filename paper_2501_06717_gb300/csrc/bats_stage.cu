@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(128) k_amr_ghost_table(const StageArgs a, cons
 // The sample of entry e (the generic point location for GT_GENERIC).
 __device__ __forceinline__ void ghost_sample_w(const StageArgs& a, const GhostTask& T, int32_t e, int tid, float w[8]) {
   if (e >= 0) {
-    const float* p = a.Win + static_cast<int64_t>((e & (GT_RESTRICT - 1)) >> 9) * (NV * NCELL) + (e & 511);
+    const int cell = e & GT_RESTRICT ? chki((e & 511) + NC * NC + NC + 1, 0, NCELL) - (NC * NC + NC + 1) : e & 511;
+    const float* p = a.Win + chk((e & (GT_RESTRICT - 1)) >> 9, 0, a.nblocks) * (NV * NCELL) + cell;
     if (e & GT_RESTRICT) {
       restrict_at(p, a.ph.gm1f, w);
     } else {
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(256) k_load_state(const double* __restrict__ e
   const GridDev& G = grids[B.grid];
   const int64_t vstride = static_cast<int64_t>(G.nb) * NCELL;
   const double* src = ext + ext_off + static_cast<int64_t>(G.block0) * (NV * NCELL) +
-                      static_cast<int64_t>(blk - G.block0) * NCELL;
+                      chk(blk - G.block0, 0, G.nb) * NCELL;
   const int64_t base = static_cast<int64_t>(blk) * (NV * NCELL);
   double u[2][8];
 #pragma unroll
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(256) k_store_state(const double* __restrict__ 
   const GridDev& G = grids[blocks[blk].grid];
   const int64_t vstride = static_cast<int64_t>(G.nb) * NCELL;
   double* dst = ext + ext_off + static_cast<int64_t>(G.block0) * (NV * NCELL) +
-                static_cast<int64_t>(blk - G.block0) * NCELL + threadIdx.x;
+                chk(blk - G.block0, 0, G.nb) * NCELL + threadIdx.x;
   const double* src = U + static_cast<int64_t>(blk) * (NV * NCELL) + threadIdx.x;
   double u[16];
 #pragma unroll

@@ -1827,10 +1827,10 @@ __device__ __forceinline__ void faces_mx(const int D, const StageArgs& a, const 
 }
 
 // Mixed plain kernel, common case (first or second midpoint stage with the
-// global dt, no body cell in the block, no B0): the cell phase on the first
-// 256 threads, two cells each -- cell c and cell c + 256 (the same (i, j),
-// four layers apart in k) -- with the FP32 work packed over the pair and the
-// FP64 accumulation per cell.  The same arithmetic, value for value, as the
+// global dt, no body cell in the block, no B0): two cells per thread, cell c
+// (0..255, eight parts of 32) and cell c + 256 (the same (i, j), four layers
+// apart in k), with the FP32 work packed over the pair and the FP64
+// accumulation per cell.  The same arithmetic, value for value, as the
 // general cell phase (which runs the other cases, one cell per thread).
 // Returns this thread's largest CFL bound (last stage), 0 otherwise.
 // The pair's primitives Wc (the stage input) come from the tile, read by the
@@ -1838,19 +1838,18 @@ __device__ __forceinline__ void faces_mx(const int D, const StageArgs& a, const 
 // last stage reads them, for the Powell term, from memory); the grid's dt is
 // loaded by the caller ahead of the wait for the faces.
 __device__ __forceinline__ void cells_mx_pair_w(const float* sT, int tid, float2 Wc[8]) {
-  if (tid >= NCELL / 2) return;
-  const int cs = mx_int(tid);  // the interior's swizzle (the pair shares it)
+  const int cs = chki(mx_int(tid), 0, NCELL / 2);  // the interior's swizzle (the pair shares it)
 #pragma unroll
   for (int v = 0; v < NV; v++) Wc[v] = make_float2(sT[v * NCELL + cs], sT[v * NCELL + cs + NCELL / 2]);
 }
 __device__ __forceinline__ float cells_mx_pair(const StageArgs& a, const GridDev& G, const BlockDev& B, int blk,
                                                const float2 Wc[8], double dtg, const float* sF, int tid, float fx,
                                                float fy, float fz, float idx0, float idx1, float idx2, float gamma) {
-  if (tid >= NCELL / 2) return 0.f;
   const PhysDev& ph = a.ph;
   const int c = tid, ci = c & 7, cj = (c >> 3) & 7, ck = c >> 6;  // ck 0..3; the pair's second cell: ck + 4
-  const int tx = (ck * NC + cj) * 9 + ci, ty = (ck * NC + ci) * 9 + cj, tz = (cj * NC + ci) * 9 + ck;
   constexpr int DX = 4 * NC * 9, DZ = 4;   // face-index offsets of the second cell (x, y: +288; z: +4)
+  const int tx = chki((ck * NC + cj) * 9 + ci, 0, NFACE - DX - 1), ty = chki((ck * NC + ci) * 9 + cj, 0, NFACE - DX - 1),
+            tz = chki((cj * NC + ci) * 9 + ck, 0, NFACE - DZ - 1);
   const float* Fx = sF;
   const float* Fy = sF + 9 * NFACE;
   const float* Fz = sF + 2 * 9 * NFACE;
@@ -2245,7 +2244,7 @@ __global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constan
   const int n = items * bpi - (has_last ? nitems * bpi - a.nblocks : 0);
   auto block_of = [&](int q) {
     const int it = q / bpi;
-    return (static_cast<int>(blockIdx.x) + it * static_cast<int>(gridDim.x)) * bpi + (q - it * bpi);
+    return chki((static_cast<int>(blockIdx.x) + it * static_cast<int>(gridDim.x)) * bpi + (q - it * bpi), 0, a.nblocks);
   };
   // one thread (lane 0, whose `failed` the warp then takes over): the copies of
   // the CTA's q-th block, once its tile is free
