@@ -2337,9 +2337,9 @@ __global__ void __launch_bounds__(MX_THREADS, 1) k_stage_mx(const __grid_constan
       }
     }
     if (a.last && a.kind != 2) {
-      // this warp's largest bound: the bits of non-negative floats order like
-      // the floats
-      const uint32_t mw = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+      // this warp's largest bound: the bits of non-negative floats order like the
+      // floats (NaN, of two non-physical cells, counts as none)
+      const uint32_t mw = __reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(m, 0.f)));
       if (lane == 0 && mw != 0u)
         atomicMax(&a.smax_next[B.grid],
                   static_cast<unsigned long long>(__double_as_longlong(f2d_int(__uint_as_float(mw)))));
