@@ -39,16 +39,16 @@ METRIC = "cell-updates/s/GB300"
 UNIT = "cell-updates/s"
 BYTES_PER_CELL_UPDATE = 320  # FP64 state: stage 1 reads U^n, writes U*; stage 2 reads U*, U^n, writes U^{n+1}
 # FP64 form: executed FP64 flops per cell-update (DADD + DMUL + 2 DFMA, both
-# stages: 970 + 1,082), ncu counters of k_stage<0,...> on the first 8 grids
+# stages: 1,003 + 1,128), ncu counters of k_stage<0,...> on the first 8 grids
 # of the batched workload (profiles/k_stage_fp64_batched8_ncu.md)
-FP64_FLOPS_PER_CELL_UPDATE = 2052
+FP64_FLOPS_PER_CELL_UPDATE = 2130
 
 # DRAM traffic of one stage launch per cell, from the ncu capture summarised
 # in profiles/ (None until a capture of the current kernel source exists).
 NCU_TRAFFIC = {
     # precision: (DRAM bytes per cell per launch, mean of the two stages, sha256 of the stage
     # kernel's sources -- bats_stage_kernel.h then bats_stage.cu -- at capture)
-    "mixed": (123.0, "af3d88b1df202cbbf63044d9ed7280cb3edf65f48f1f1a394b8328928559617f"),
+    "mixed": (123.0, "15aefe02a0980cffbc75ef63932328fc35801d49be453bd39724bc0c8c2891d1"),
 }
 
 

@@ -7,8 +7,11 @@ own time of the stages) and keeps the fastest:
   blocks_per_cta blocks per work item (consecutive blocks in leaf order, which
                  is a space-filling order, so neighbours' halos hit in L2)
   ctas_per_sm    persistent CTAs per SM (0 = the occupancy limit)
-                 (the mixed form's plain stage always walks its work items with
-                 one CTA per SM: there the first two differ little)
+                 (the mixed form always walks its work items with one CTA per
+                 SM, so persistent and ctas_per_sm change nothing there, and the
+                 plain stage's items have at most as many blocks as leave a CTA
+                 eight: candidates that differ in these only are the same launch,
+                 and which of them is kept does not matter)
   staging        mixed form only: how the stage kernel stages each block's
                  padded stencil in shared memory -- 1 = the same-level face
                  slabs by tensor copies (TMA), 0 = gathered by the threads

@@ -20,7 +20,6 @@
 namespace batsk {
 
 // launchers defined next to the kernels (bats_stage.cu)
-size_t stage_smem_bytes(bool mixed);
 cudaError_t stage_setup(int occ[2]);
 cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const StageArgs& a);
 cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,
@@ -509,10 +508,12 @@ int launch_stage_one(bats_t* h, const StageArgs& a0, bool make_ghosts = true, bo
   }
   // FP64 form with at most half as many blocks as SMs: a block is FP64-bound on
   // its one SM, so 2, 4 or 8 CTAs share it, by layers of cells, as long as all of
-  // them run at once (one step of 8 blocks with its state in and out: 304 us
-  // whole, 149 us in eight parts).  A layer split computes the faces between two
-  // parts twice and every slope for both of its faces; 120 blocks in four parts
-  // on 152 SMs would take four rounds of more than a quarter.
+  // them run at once: a layer split computes the faces between two parts twice and
+  // every slope for both of its faces.  Per stage, whole and in 2, 4, 8 parts on
+  // 152 SMs: 75 blocks 111, 66, 82, 118 us; 80 blocks 111, 129, 121, 146; 120
+  // blocks 111, 130, 162, 204.  (A last round that is nearly empty can be split
+  // with gain too, 153 to 228 blocks 219 whole, 193 in halves; 306 blocks 328 and
+  // 320; 250 blocks lose, 220 and 257.  The rule leaves those whole.)
   if (!mixed && !a.learned && a.kind < 3) {
     a.parts = 8;
     while (a.parts > 1 && a.nblocks * a.parts > h->num_sms) a.parts /= 2;

@@ -147,10 +147,11 @@ struct StageArgs {
   float* Xf;              // kind 4: FP32 features, 40 per face
   double* Fd;             // kind 4: plain Rusanov flux (8, x/y/z components), rho_ref, c_ref per face
   const float* Y;         // normalised correction in the face frame, 8 per face
-  // mixed form, plain stage kernel: tensor maps of Win (interior box
-  // 8x8x8x8 with the 32-byte swizzle; face-slab boxes 4x8x8x8, 8x2x8x8,
-  // 8x8x2x8 over the dims (i, j, k, 8 * block + v)), and the staging layout:
-  // 1 = same-level face slabs by tensor copies, 0 = gathered by the threads
+  // mixed form, plain stage kernel: tensor maps of Win (tm[0]: the interior, box
+  // 32x2x8x8 with the 128-byte swizzle over the dims (four rows of i, j / 4, k,
+  // 8 * block + v); tm[1..3]: face-slab boxes 4x8x8x8, 8x2x8x8, 8x8x2x8 over the
+  // dims (i, j, k, 8 * block + v)), and the staging layout: 1 = same-level face
+  // slabs by tensor copies, 0 = gathered by the threads
   int32_t stage_tma;
   int32_t gbuf_mx;        // ghost-slab buffer in the mixed tile's slab layouts (1) or the generic one (0)
   MlpDev mlp;             // mixed learned stage: the network, run fused in the stage kernel

@@ -322,7 +322,8 @@ __device__ __forceinline__ void pack_param(const MlpDev& m, int e, float p) {
 // gradient (the partials in CTA order, as k_mlp_grad_reduce), Adam (Kingma & Ba
 // 2015) on the FP32 master weight, bias-corrected, and the BF16 copies.  Three
 // launches (sum, update, copies) made up a third of a step: 14 steps of 8,192
-// samples with four launches each took 709 us, with two 488 us.  CTAs of 64 threads: the sums are chains of loads, spread over the SMs.
+// samples with four launches each took 709 us, with two 488 us.  CTAs of 64
+// threads: the sums are chains of loads, spread over the SMs.
 __global__ void __launch_bounds__(64) k_mlp_update(const float* __restrict__ partial,
                                                    const double* __restrict__ partial_loss, int nparts,
                                                    double* __restrict__ loss, float* __restrict__ p,

@@ -23,7 +23,6 @@
 #include "bats_internal.h"
 
 namespace batsk {
-size_t stage_smem_bytes(bool mixed);
 cudaError_t stage_setup(int occ[2]);
 cudaError_t launch_stage_kernel(bool mixed, int grid, cudaStream_t st, const StageArgs& a);
 cudaError_t launch_load_state(bool mixed, const double* ext, int64_t ext_off, double* U, float* W, const GridDev* grids,

@@ -139,9 +139,6 @@ __global__ void __launch_bounds__(128) k_amr_ghosts(const StageArgs a, const Gho
 }
 
 // ---------------------------------------------------------------------------
-// The fused stage kernel.
-
-// ---------------------------------------------------------------------------
 // Small kernels.
 
 // Conservative inflow/body states (and the mixed-form primitives of the inflow).
@@ -600,9 +597,6 @@ __global__ void k_debug_fp64_ops(const double* in, int n, double* out) {
 // ---------------------------------------------------------------------------
 // Host-side launchers (kernel stubs stay in this translation unit).
 
-size_t stage_smem_bytes(bool mixed) {
-  return mixed ? StageCfg<true>::SMEM : StageCfg<false>::SMEM;
-}
 // dynamic shared memory of a stage kernel: the mixed plain kernel stages
 // its own tile layout
 static size_t stage_smem(bool mixed, bool lrn) {

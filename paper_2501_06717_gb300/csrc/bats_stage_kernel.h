@@ -1182,12 +1182,12 @@ __device__ __forceinline__ void b0_cell(const StageArgs& a, const GridDev& G, co
 // ---------------------------------------------------------------------------
 // FP64 form, plain faces.  GB300 runs FP64 at 1/64 of the FP32 rate, so this
 // code is written for the fewest FP64 operations: selections and limiters on
-// bit patterns (integer pipe), roots by rsqrt64_est, no division, no operation
-// on an absent B0, face values stored doubled (the cell phase halves its
-// spacing instead).  Together with the warp-wise halves of faces64: 120 blocks
-// 561 -> 290 us a step, one step of 8 blocks with its state in and out 527 ->
-// 322 us, six grids with the HLL flux 36.7 -> 23.0 ms; the FP64 pipe is 81 to
-// 83 % busy before and after: the time went with the operations.
+// bit patterns (integer pipe), roots by rsqrt64_est, no division within the usual
+// range, no operation on an absent B0, face values stored doubled (the cell phase
+// halves its spacing instead).  With divisions, the general roots and comparisons
+// 120 blocks took 561 us a step and two steps of six grids with the HLL flux 36.7
+// ms; now 282 us and 21.4 ms.  The FP64 pipe is about 80 % busy either way: the
+// time went with the operations.
 
 // The limited slope of a cell as value and factor: half the slope is f v.
 // Minmod: the difference of smaller magnitude, f = 1/2; MC (beta = 2): that
@@ -2182,15 +2182,16 @@ __device__ __forceinline__ float cells_mx_general(const StageArgs& a, const Grid
 // barriers (two CTAs per SM), the schedulers issued on 47-55 % of the cycles,
 // the cells taking as long as the faces on two thirds of the warps.  Here the
 // warps are specialised, so that the phases of neighbouring blocks overlap and
-// the copies run a block ahead: 61 % of the cycles; 8 grids (3.1 M cells), stage
-// 1 169 -> 147 us, stage 2 (FP64 accumulation) 216 -> 178 us.
+// the copies run a block ahead: 62 % of the cycles; 8 grids (3.1 M cells), stage
+// 1 165 -> 135 us, stage 2 (FP64 accumulation) 211 -> 164 us.  (With a background
+// field the 80 registers spill, some 300 bytes per thread.)
 //  * 12 face warps: faces_mx of one block after the other;
 //  * 12 cell warps: the cells of the blocks before, 1/8 of a block at a time in
 //    turn (a block's eight parts go to eight of the warps, the next block's to
 //    the other four and on): with eight warps a block's cells took twice as long
 //    as its faces in the last stage (long chains of shared-memory loads, FP64
-//    operations at 64 cycles per warp and global loads).  The warp with a block's first part also issues the copies of the
-//    next block's record and tile.
+//    operations at 64 cycles per warp and global loads).  The warp with a block's
+//    first part also issues the copies of the next block's record and tile.
 // Tile q & 1 and face values q & 1 belong to the CTA's q-th block; they are
 // handed over through mbarriers: full (copies landed; faces done by the 12
 // warps) and empty (tile read by the 12 face warps and the 8 parts; face values
@@ -2524,13 +2525,13 @@ __device__ __forceinline__ bool lrn_network(LrnSmem& s, const uint4 xrow[6], flo
 }
 
 // The fused stage of the FP64 form and of the learned correction in the mixed form
-// (the plain mixed one: k_stage_mx below), one CTA of 384 threads per SM.  Per
-// block: (1) interior by TMA, face-slab ghosts by threads; (2) FP64 form: primitives in place; (3) faces of all
-// three directions at once on the first FACE_THREADS threads, two per grid
-// line (faces 0-4 and 5-8), each sliding a window along its line so that
-// every cell is loaded and every limited slope computed once; (4) per cell:
-// flux differences x, y, z, the sources, the update and (last stage) the CFL
-// bound.
+// (the plain mixed one: k_stage_mx above), one CTA of 384 threads per SM.  Per
+// block: (1) interior by TMA, face-slab ghosts by threads; (2) FP64 form:
+// primitives in place; (3) faces of all three directions at once on the first
+// FACE_THREADS threads, two per grid line (faces 0-4 and 5-8), each sliding a
+// window along its line so that every cell is loaded and every limited slope
+// computed once; (4) per cell: flux differences x, y, z, the sources, the update
+// and (last stage) the CFL bound.
 template <bool MIXED, int LIM, bool HAS_B0, bool LRN, int FLX>
 __global__ void __launch_bounds__(STAGE_THREADS, 1) k_stage(const __grid_constant__ StageArgs a) {
   static_assert(!MIXED || LRN, "the plain mixed stage is k_stage_mx");
